@@ -66,6 +66,17 @@ struct lowd_ctx {
     float* l = nullptr;        // [n + 1] loads; slot n is the padding sentinel
     float* l_lo = nullptr;     // [n + 1] low parts: the load is l + l_lo (pair arithmetic in the sweep)
 
+    // systolic passes (schedule 1): the plain edges' splits and weights in a dense array; the
+    // class-major arrays above then hold the star edges only
+    int sys = 0;               // 1: the plain edges are in the cells
+    int sys_pair = 0;          // 1: loads as FP32 pairs during the passes, 0: single FP32
+    int64_t sys_m = 0;         // plain edges
+    float* sys_cs = nullptr;   // cells: splits
+    float* sys_cw = nullptr;   // cells: weights (weighted only)
+    int32_t* sys_ids = nullptr;  // [sys_m] plain edge ids (null: every edge)
+    ulonglong2* sys_streams = nullptr;  // column streams between blocks, entries (hi, tag), (lo, tag)
+    uint32_t sys_tag = 0;      // next free tag (0: streams not cleared yet)
+
     // streamed schedule (2): chunked class-major stream, loads in global memory
     int32_t s2_NC = 0, s2_E = 0, s2_S = 0, s2_D = 0;   // chunks, edges per stage, stages, lead
     int32_t s2_K = 0;             // leading classes run as grid-wide steps
@@ -174,6 +185,16 @@ lowd_status lowd_sweep_rederive(lowd_ctx* h, double* stats3);
 lowd_status lowd_sweep_splits_canonical(lowd_ctx* h, float* out_dev);
 lowd_status lowd_sweep_load_canonical(lowd_ctx* h, const float* splits_dev);
 lowd_status lowd_sweep_edge_order(lowd_ctx* h, int32_t* out_dev);
+
+// systolic.cu
+bool lowd_sys_serves(int32_t n, int64_t m, int32_t C, bool pair);
+lowd_status lowd_sys_class_sizes(lowd_ctx* h, const int32_t* u, const int32_t* v, int64_t m, int32_t* cnt_h);
+lowd_status lowd_sys_build(lowd_ctx* h, const int32_t* plain_ids, int64_t m_plain, const float* init_splits_canon);
+lowd_status lowd_sys_rederive(lowd_ctx* h, double* L64);
+lowd_status lowd_sys_to_canonical(lowd_ctx* h, float* out);
+lowd_status lowd_sys_from_canonical(lowd_ctx* h, const float* in);
+lowd_status lowd_sys_edge_order(lowd_ctx* h, int32_t* out);
+cudaError_t lowd_sys_passes(lowd_ctx* h, int32_t passes);
 
 // stars.cu
 struct StarSplit {

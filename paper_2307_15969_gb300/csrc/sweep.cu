@@ -28,6 +28,8 @@
 #include "prims.cuh"
 #include "async.cuh"
 
+#include <vector>
+
 using namespace lowd;
 
 namespace {
@@ -411,6 +413,7 @@ constexpr int kTmaMaxStages = 16;
 constexpr int kStoreSlack = 1;    // bulk stores allowed to be still reading their stage
 constexpr int kStoreGroups = 8;   // bulk stores allowed in flight at all
 constexpr uint32_t kWaitLimit = 1u << 22;   // try_wait rounds before giving up
+constexpr int32_t kTmaMinClasses = 369;     // fewest classes it runs on (16 per chunk, 16 stages)
 
 struct TmaLayout {
     uint32_t bars, L, CO, stages, stage_bytes, arr_bytes, total;
@@ -878,31 +881,55 @@ k_sweep_simple(int32_t n, int32_t C, const int32_t* __restrict__ coff, const uin
     }
 }
 
-template <bool WEIGHTED>
-cudaError_t launch_sweep_tma(lowd_ctx* h, int32_t passes, int32_t maxlen, bool* launched) {
-    *launched = false;
-    const size_t budget = 227 * 1024;
-    // chunk size G (classes per staged copy) and stage count S: the largest G whose
-    // chunks leave room for at least kMinStages stages, then as many stages as fit
-    constexpr int kMinStages = 3;
+// Chunk size G (classes per staged copy) and stage count S of the staged sweep: the largest G
+// whose chunks leave room for at least kMinStages stages, then as many stages as fit.  G = 0 if
+// it cannot run.
+struct TmaPick {
     int32_t G = 0, S = 0, chunk = 0;
     TmaLayout lay{};
+};
+
+TmaPick tma_pick(const lowd_ctx* h, bool weighted) {
+    constexpr size_t budget = 227 * 1024;
+    constexpr int kMinStages = 3;
+    TmaPick p;
     for (int32_t g : {16, 8, 4, 2, 1}) {
         int32_t mx = 0;  // longest chunk of g classes
         for (int32_t c0 = 0; c0 < h->C; c0 += g) mx = max(mx, h->coff_h[min(c0 + g, h->C)] - h->coff_h[c0]);
         int32_t s = kTmaMaxStages;
-        TmaLayout t = tma_layout(h->n, h->C, s, mx, WEIGHTED, g);
-        while (s > kMinStages && t.total > budget) t = tma_layout(h->n, h->C, --s, mx, WEIGHTED, g);
-        if (t.total <= budget) { G = g; S = s; chunk = mx; lay = t; break; }
+        TmaLayout t = tma_layout(h->n, h->C, s, mx, weighted, g);
+        while (s > kMinStages && t.total > budget) t = tma_layout(h->n, h->C, --s, mx, weighted, g);
+        if (t.total <= budget) { p.G = g; p.S = s; p.chunk = mx; p.lay = t; break; }
     }
-    if (G == 0) return cudaSuccess;
-    const int32_t NC = (h->C + G - 1) / G;
+    if (p.G == 0) return p;
+    const int32_t NC = (h->C + p.G - 1) / p.G;
     // a chunk's splits are re-read one pass later: its store must be older than the
     // kStoreGroups stores allowed in flight when the producer loads it again
-    if (NC < S - kStoreSlack + kStoreGroups + 1) return cudaSuccess;
-    // edges per consumer thread: enough warps to hide latency, few enough to keep the
-    // per-class bookkeeping small
-    const int E = maxlen > 2 * kTmaConsumers ? 4 : (maxlen > kTmaConsumers ? 2 : 1);
+    if (NC < p.S - kStoreSlack + kStoreGroups + 1) p.G = 0;
+    return p;
+}
+
+int32_t longest_class(const lowd_ctx* h) {
+    int32_t maxlen = 0;
+    for (int32_t c = 0; c < h->C; ++c) maxlen = max(maxlen, h->coff_h[c + 1] - h->coff_h[c]);
+    return maxlen;
+}
+
+// Edges per consumer thread of the staged sweep: enough warps to hide latency, few enough to keep
+// the per-class bookkeeping small.
+int tma_edges_per_thread(int32_t maxlen) {
+    return maxlen > 2 * kTmaConsumers ? 4 : (maxlen > kTmaConsumers ? 2 : 1);
+}
+
+template <bool WEIGHTED>
+cudaError_t launch_sweep_tma(lowd_ctx* h, int32_t passes, int32_t maxlen, bool* launched) {
+    *launched = false;
+    const TmaPick pick = tma_pick(h, WEIGHTED);
+    if (pick.G == 0) return cudaSuccess;
+    const int32_t G = pick.G, S = pick.S, chunk = pick.chunk;
+    const TmaLayout& lay = pick.lay;
+    const int32_t NC = (h->C + G - 1) / G;
+    const int E = tma_edges_per_thread(maxlen);
     int threads = ((((maxlen + E - 1) / E) + 31) / 32) * 32;
     if (threads < 64) threads = 64;
     if (threads > kTmaConsumers) threads = kTmaConsumers;
@@ -955,29 +982,40 @@ void sweep_ranks(lowd_ctx* h) {
     dfree(h, &ok[0]); dfree(h, &ok[1]); dfree(h, &ov[0]); dfree(h, &ov[1]);
 }
 
-template <bool WEIGHTED>
-cudaError_t launch_sweep_flow(lowd_ctx* h, int32_t passes, int32_t maxlen, bool* launched) {
-    *launched = false;
-    if (maxlen > kTmaConsumers) return cudaSuccess;
-    if (!h->crk) sweep_ranks(h);
-    if (!h->crk) return cudaSuccess;
-    const size_t budget = 227 * 1024;
-    constexpr int kMinStages = 3;
+struct FlowPick {
     int32_t G = 0, S = 0, chunk = 0;
     FlowLayout lay{};
+};
+
+FlowPick flow_pick(const lowd_ctx* h, bool weighted, int32_t maxlen) {
+    constexpr size_t budget = 227 * 1024;
+    constexpr int kMinStages = 3;
+    FlowPick p;
+    if (maxlen > kTmaConsumers) return p;
     for (int32_t g : {16, 8, 4, 2, 1}) {
         int32_t mx = 0;
         for (int32_t c0 = 0; c0 < h->C; c0 += g) mx = max(mx, h->coff_h[min(c0 + g, h->C)] - h->coff_h[c0]);
         int32_t s = kTmaMaxStages;
-        FlowLayout t = flow_layout(h->n, h->C, s, mx, WEIGHTED, g);
-        while (s > kMinStages && t.total > budget) t = flow_layout(h->n, h->C, --s, mx, WEIGHTED, g);
+        FlowLayout t = flow_layout(h->n, h->C, s, mx, weighted, g);
+        while (s > kMinStages && t.total > budget) t = flow_layout(h->n, h->C, --s, mx, weighted, g);
         if (t.total > budget) continue;
         const int32_t NC = (h->C + g - 1) / g;
         if (NC < s - kStoreSlack + kStoreGroups + 1) continue;   // split store ordering, as k_sweep_tma
-        G = g; S = s; chunk = mx; lay = t;
+        p.G = g; p.S = s; p.chunk = mx; p.lay = t;
         break;
     }
-    if (G == 0) return cudaSuccess;
+    return p;
+}
+
+template <bool WEIGHTED>
+cudaError_t launch_sweep_flow(lowd_ctx* h, int32_t passes, int32_t maxlen, bool* launched) {
+    *launched = false;
+    const FlowPick pick = flow_pick(h, WEIGHTED, maxlen);
+    if (pick.G == 0) return cudaSuccess;
+    if (!h->crk) sweep_ranks(h);
+    if (!h->crk) return cudaSuccess;
+    const int32_t G = pick.G, S = pick.S, chunk = pick.chunk;
+    const FlowLayout& lay = pick.lay;
     const int32_t NC = (h->C + G - 1) / G;
     int threads = ((maxlen + 31) / 32) * 32;
     if (threads < 64) threads = 64;
@@ -1003,8 +1041,7 @@ cudaError_t launch_sweep_flow(lowd_ctx* h, int32_t passes, int32_t maxlen, bool*
 template <bool WEIGHTED>
 cudaError_t launch_sweep(lowd_ctx* h, int32_t passes) {
     {
-        int32_t maxlen = 0;
-        for (int32_t c = 0; c < h->C; ++c) maxlen = max(maxlen, h->coff_h[c + 1] - h->coff_h[c]);
+        const int32_t maxlen = longest_class(h);
         bool launched = false;
         cudaError_t e = cudaSuccess;
         if (h->use_versions) {
@@ -1046,16 +1083,27 @@ cudaError_t launch_sweep(lowd_ctx* h, int32_t passes) {
     return cudaGetLastError();
 }
 
+// Passes over the plain edges (schedule 1): the systolic array where it holds them, else the
+// one-CTA kernels.
+cudaError_t run_plain(lowd_ctx* h, int32_t passes) {
+    if (h->sys) {
+        h->sweep_kernel = h->sys_pair ? 1 : 2;
+        h->sweep_E = h->sys_pair ? tma_edges_per_thread(longest_class(h)) : 0;
+        return lowd_sys_passes(h, passes);
+    }
+    return h->cw ? launch_sweep<true>(h, passes) : launch_sweep<false>(h, passes);
+}
+
 cudaError_t run_passes(lowd_ctx* h, int32_t passes) {
     if (passes <= 0 || h->m == 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(h->d_i32 + 8, 0, sizeof(int32_t), h->st);
     if (e != cudaSuccess) return e;
     if (h->sched == 2) return lowd_stream_passes(h, passes);
-    if (h->star_S == 0) return h->cw ? launch_sweep<true>(h, passes) : launch_sweep<false>(h, passes);
+    if (h->star_S == 0) return run_plain(h, passes);
     // hub stars: per pass, the plain classes, then the star steps
     e = cudaMemsetAsync(h->d_i32 + 12, 0, 2 * sizeof(int32_t), h->st);   // grid barrier words
     for (int32_t t = 0; t < passes && e == cudaSuccess; ++t) {
-        if (h->C > 0) e = h->cw ? launch_sweep<true>(h, 1) : launch_sweep<false>(h, 1);
+        if (h->C > 0) e = run_plain(h, 1);
         if (e == cudaSuccess) e = lowd_star_pass(h);
     }
     return e;
@@ -1063,9 +1111,92 @@ cudaError_t run_passes(lowd_ctx* h, int32_t passes) {
 
 }  // namespace
 
-// Build the schedule and the class-major streams, then initialise the splits (equal
-// split, or the given canonical-order splits) and the loads.
+// The schedule as the systolic array holds it, if it serves these edges (*built): class sizes
+// and offsets, the cells, and the class-major arrays for the star edges alone.  The loads are
+// pairs exactly where the staged sweep would run (single FP32 loads otherwise, as in the
+// register-ring sweep), so the results do not depend on which kernel runs a graph.
+static lowd_status prepare_systolic(lowd_ctx* h, const StarSplit& sp, const float* init_splits_canon, bool* built) {
+    cudaStream_t st = h->st;
+    *built = false;
+    const int64_t mc = sp.pid ? sp.m_plain : h->m;
+    if (mc == 0 || h->use_versions) return LOWD_OK;
+    const int32_t P = h->n + (h->n & 1) - 1;
+    // no need to count the classes of a graph that would not be served with half of them
+    if (!lowd_sys_serves(h->n, mc, P / 2, P > 2 * kTmaMinClasses)) return LOWD_OK;
+    std::vector<int32_t> cnt((size_t)P), real;
+    LOWD_TRY(lowd_sys_class_sizes(h, sp.pid ? sp.gu : h->u, sp.pid ? sp.gv : h->v, mc, cnt.data()));
+    real.reserve((size_t)P + 1);
+    real.push_back(0);
+    for (int32_t c = 0; c < P; ++c)
+        if (cnt[(size_t)c]) real.push_back(real.back() + cnt[(size_t)c]);
+    const int32_t C = (int32_t)real.size() - 1;
+    if (C < (h->w ? kRingW : kRingU)) return LOWD_OK;
+    h->coff_h = (int32_t*)malloc(sizeof(int32_t) * ((size_t)C + 1));
+    if (!h->coff_h) return LOWD_ERR_OUT_OF_MEMORY;
+    h->coff_h[0] = 0;   // offsets of the classes padded to a multiple of 4 edges
+    for (int32_t c = 0; c < C; ++c)
+        h->coff_h[c + 1] = h->coff_h[c] + ((real[(size_t)c + 1] - real[(size_t)c] + 3) & ~3);
+    h->C = C;
+    h->sys_pair = tma_pick(h, h->w != nullptr).G > 0 ? 1 : 0;
+    const bool serves = lowd_sys_serves(h->n, mc, C, h->sys_pair != 0);
+    const lowd_status b = serves ? lowd_sys_build(h, sp.pid, mc, init_splits_canon) : LOWD_ERR_OUT_OF_MEMORY;
+    if (b != LOWD_OK) {   // not served, or no memory for the cells: the class-major kernels need less
+        dfree(h, &h->sys_cs); dfree(h, &h->sys_cw); dfree(h, &h->sys_ids);
+        free(h->coff_h);
+        h->coff_h = nullptr;
+        h->C = 0;
+        return b == LOWD_ERR_OUT_OF_MEMORY ? LOWD_OK : b;
+    }
+    LOWD_TRY(dalloc(h, &h->coff_real, (size_t)C + 1));
+    LOWD_CK(cudaMemcpyAsync(h->coff_real, real.data(), sizeof(int32_t) * real.size(), cudaMemcpyHostToDevice, st));
+    h->m_pad = sp.ms;
+    LOWD_TRY(dalloc(h, &h->perm, sp.ms));
+    LOWD_TRY(lowd_star_blocks(h, sp, 0, C, mc));
+    LOWD_TRY(dalloc(h, &h->cuv, sp.ms));
+    if (h->w) LOWD_TRY(dalloc(h, &h->cw, sp.ms));
+    LOWD_TRY(dalloc(h, &h->cs, sp.ms));
+    if (sp.ms > 0)
+        LOWD_LAUNCH(k_gather_streams, grid_for(sp.ms), kT, 0, st, h->perm, sp.ms, h->n, h->u, h->v, h->w,
+                    init_splits_canon, h->cuv, h->cw, h->cs);
+    LOWD_CK_LAUNCH();
+    LOWD_CK(cudaStreamSynchronize(st));   // `real` leaves scope
+    h->sys = 1;
+    *built = true;
+    return LOWD_OK;
+}
+
+static lowd_status prepare_schedule(lowd_ctx* h, int schedule_req, const float* init_splits_canon, bool systolic);
+
+// Per-node versions (kernel 5) read the class-major arrays: a graph held in the systolic array
+// moves there, once, keeping its splits (its loads are re-derived from them, as after every call).
+static lowd_status leave_systolic(lowd_ctx* h) {
+    float* s = nullptr;
+    LOWD_TRY(dalloc(h, &s, h->m));
+    lowd_status r = lowd_sweep_splits_canonical(h, s);
+    if (r == LOWD_OK) {
+        dfree(h, &h->sys_cs); dfree(h, &h->sys_cw); dfree(h, &h->sys_ids); dfree(h, &h->sys_streams);
+        dfree(h, &h->perm); dfree(h, &h->coff); dfree(h, &h->coff_real); dfree(h, &h->cuv);
+        dfree(h, &h->cw); dfree(h, &h->cs); dfree(h, &h->l); dfree(h, &h->l_lo);
+        dfree(h, &h->star_step_seg); dfree(h, &h->star_seg_beg); dfree(h, &h->star_seg_hub); dfree(h, &h->star_bbuf);
+        free(h->coff_h);
+        h->coff_h = nullptr;
+        h->sys = 0;
+        h->sys_m = 0;
+        h->inited = 0;
+        r = prepare_schedule(h, 1, s, false);
+    }
+    cudaStreamSynchronize(h->st);
+    dfree(h, &s);
+    return r;
+}
+
+// Build the schedule and its arrays, then initialise the splits (equal split, or the given
+// canonical-order splits) and the loads.
 lowd_status lowd_sweep_prepare(lowd_ctx* h, int schedule_req, const float* init_splits_canon) {
+    return prepare_schedule(h, schedule_req, init_splits_canon, true);
+}
+
+static lowd_status prepare_schedule(lowd_ctx* h, int schedule_req, const float* init_splits_canon, bool systolic) {
     cudaStream_t st = h->st;
     const int64_t m = h->m;
     const int32_t n = h->n;
@@ -1090,6 +1221,19 @@ lowd_status lowd_sweep_prepare(lowd_ctx* h, int schedule_req, const float* init_
     };
     do {
         if ((s = lowd_star_split(h, h->hub_tau, 1, &sp))) break;
+        if (systolic) {
+            bool built = false;
+            if ((s = prepare_systolic(h, sp, init_splits_canon, &built))) break;
+            if (built) {
+                if ((s = dalloc(h, &h->l, (size_t)n + 1))) break;
+                if ((s = dalloc(h, &h->l_lo, (size_t)n + 1))) break;
+                h->sched = 1;
+                h->inited = 1;
+                double st3[3];
+                s = lowd_sweep_rederive(h, st3);
+                break;
+            }
+        }
         const int64_t mc = sp.pid ? sp.m_plain : m;   // edges the colouring covers
         const int32_t* cu = sp.pid ? sp.gu : h->u;
         const int32_t* cv = sp.pid ? sp.gv : h->v;
@@ -1178,7 +1322,11 @@ lowd_status lowd_sweep_rederive(lowd_ctx* h, double* stats3) {
     if (h->sched == 2) {
         lowd_status r = lowd_stream_rederive(h, L64);
         if (r != LOWD_OK) { dfree(h, &L64); return r; }
-    } else if (h->m_pad > 0) {
+    } else if (h->sys) {
+        lowd_status r = lowd_sys_rederive(h, L64);
+        if (r != LOWD_OK) { dfree(h, &L64); return r; }
+    }
+    if (h->sched != 2 && h->m_pad > 0) {
         LOWD_LAUNCH(k_rederive, grid_for(h->m_pad), kT, 0, st, h->m_pad, h->cuv, h->cw, h->cs, L64);
     }
     LOWD_LAUNCH(k_load_stats, grid_for(h->n), kT, 0, st, L64, h->n, h->l, h->l_lo, h->d_stats);
@@ -1193,6 +1341,7 @@ lowd_status lowd_sweep_rederive(lowd_ctx* h, double* stats3) {
 }
 
 lowd_status lowd_sweep_splits_canonical(lowd_ctx* h, float* out_dev) {
+    if (h->sys) LOWD_TRY(lowd_sys_to_canonical(h, out_dev));
     if (h->m_pad > 0)
         LOWD_LAUNCH(k_splits_to_canonical, grid_for(h->m_pad), kT, 0, h->st, h->perm, h->m_pad, h->cs, out_dev);
     LOWD_CK_LAUNCH();
@@ -1200,6 +1349,7 @@ lowd_status lowd_sweep_splits_canonical(lowd_ctx* h, float* out_dev) {
 }
 
 lowd_status lowd_sweep_load_canonical(lowd_ctx* h, const float* splits_dev) {
+    if (h->sys) LOWD_TRY(lowd_sys_from_canonical(h, splits_dev));
     if (h->m_pad > 0)
         LOWD_LAUNCH(k_splits_from_canonical, grid_for(h->m_pad), kT, 0, h->st, h->perm, h->m_pad, splits_dev, h->cs);
     LOWD_CK_LAUNCH();
@@ -1208,6 +1358,14 @@ lowd_status lowd_sweep_load_canonical(lowd_ctx* h, const float* splits_dev) {
 
 // The update order as canonical edge ids (padding removed) into out_dev [m].
 lowd_status lowd_sweep_edge_order(lowd_ctx* h, int32_t* out_dev) {
+    if (h->sys) {   // the plain classes, then the star edges (no padding)
+        LOWD_TRY(lowd_sys_edge_order(h, out_dev));
+        if (h->m_pad > 0)
+            LOWD_CK(cudaMemcpyAsync(out_dev + h->sys_m, h->perm, sizeof(int32_t) * (size_t)h->m_pad,
+                                    cudaMemcpyDeviceToDevice, h->st));
+        LOWD_CK(cudaStreamSynchronize(h->st));
+        return LOWD_OK;
+    }
     int32_t *f = nullptr, *pos = nullptr;
     LOWD_TRY(h->need_tmp(lowd_sort_tmp_bytes(h->m_pad)));
     LOWD_TRY(dalloc(h, &f, h->m_pad));
@@ -1238,6 +1396,9 @@ lowd_status lowd_sweep_run(lowd_ctx* h, int32_t k, const lowd_options* opt, lowd
     const int32_t R = o.rederive_every == 0 ? 50 : (o.rederive_every < 0 ? 0x7fffffff : o.rederive_every);
     int32_t since = 0;        // passes since the loads were last re-derived from the splits
     int32_t since_check = 0;  // passes since the last check
+    if (h->sys && h->use_versions && k > 0 && lowd_max_degree(h) < 0x7fff &&
+        flow_pick(h, h->w != nullptr, longest_class(h)).G > 0)
+        LOWD_TRY(leave_systolic(h));
     while (done < k) {
         int32_t step = k - done;
         if (o.check_every > 0 && o.check_every - since_check < step) step = o.check_every - since_check;
