@@ -81,6 +81,7 @@ void free_all(lowd_ctx* h) {
     dfree(h, &h->cw); dfree(h, &h->cs); dfree(h, &h->l); dfree(h, &h->l_lo);
     dfree(h, &h->s2_ctab); dfree(h, &h->s2_beg); dfree(h, &h->s2_ea); dfree(h, &h->s2_eb);
     dfree(h, &h->s2_srcA); dfree(h, &h->s2_srcB); dfree(h, &h->s2_lp); dfree(h, &h->s2_blob); dfree(h, &h->s2_blobo);
+    dfree(h, &h->s2_prev); dfree(h, &h->s2_nodes);
     dfree(h, &h->sys_cs); dfree(h, &h->sys_cw); dfree(h, &h->sys_ids); dfree(h, &h->sys_streams);
     dfree(h, &h->star_step_seg); dfree(h, &h->star_seg_beg); dfree(h, &h->star_seg_hub); dfree(h, &h->star_bbuf);
     if (h->tmp) cudaFree(h->tmp);   // the sort scratch is a plain allocation (need_tmp)

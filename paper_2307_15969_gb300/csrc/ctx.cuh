@@ -79,7 +79,10 @@ struct lowd_ctx {
 
     // streamed schedule (2): chunked class-major stream, loads in global memory
     int32_t s2_NC = 0, s2_E = 0, s2_S = 0, s2_D = 0;   // chunks, edges per stage, stages, lead
-    int32_t s2_K = 0;             // leading classes run as grid-wide steps
+    int32_t s2_K = 0;             // leading classes run over all SMs
+    int32_t s2_seg[2] = {0, 0};  // their launches: positions where the segments end
+    uint2* s2_prev = nullptr;     // per leading position: 1 + the position of the update before, per end
+    ulonglong2* s2_nodes = nullptr;    // [n] tagged loads (hi, tag), (lo, tag) of the leading classes
     int32_t s2_tail = 0;          // 1 if classes remain for the chunked stream
     int32_t* s2_ctab = nullptr;   // [NC][20] chunk headers
     int32_t* s2_beg = nullptr;    // [NC + 1] padded chunk begins

@@ -95,29 +95,29 @@ __global__ void k_adj_entries(const int32_t* __restrict__ ord, int64_t m, const 
 }
 
 // Entries sorted by node (stable, so by rank inside a node).  For entry j of node x holding
-// rank k: the successor of k at x is the next entry's rank; k has a predecessor at x unless
-// j is x's first entry.  side: 0 for the edge's u end, 1 for its v end.
+// rank k: the successor of k at x is the next entry's rank, its predecessor the entry before's
+// (-1: none).  side: 0 for the edge's u end, 1 for its v end.
 __global__ void k_successors(const uint32_t* __restrict__ node, const int32_t* __restrict__ rk, int64_t N,
                              const int32_t* __restrict__ ord, const int32_t* __restrict__ u,
-                             int32_t* __restrict__ succ, uint8_t* __restrict__ has_pred) {
+                             int32_t* __restrict__ succ, int32_t* __restrict__ pred) {
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < N;
          j += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t x = node[j];
         const int32_t k = rk[j];
         const int side = (u[ord[k]] == (int32_t)x) ? 0 : 1;
         succ[2 * (int64_t)k + side] = (j + 1 < N && node[j + 1] == x) ? rk[j + 1] : -1;
-        has_pred[2 * (int64_t)k + side] = (j > 0 && node[j - 1] == x) ? 1 : 0;
+        pred[2 * (int64_t)k + side] = (j > 0 && node[j - 1] == x) ? rk[j - 1] : -1;
     }
 }
 
 // pending predecessors per rank; ranks with none form the first frontier
-__global__ void k_pending(const uint8_t* __restrict__ has_pred, int64_t m, int32_t* __restrict__ pend,
+__global__ void k_pending(const int32_t* __restrict__ pred, int64_t m, int32_t* __restrict__ pend,
                           int32_t* __restrict__ frontier, int32_t* __restrict__ fcount) {
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < m; base += (int64_t)gridDim.x * blockDim.x) {
         const int64_t k = base + threadIdx.x;
         int p = 1;
         if (k < m) {
-            p = has_pred[2 * k] + has_pred[2 * k + 1];
+            p = (pred[2 * k] >= 0 ? 1 : 0) + (pred[2 * k + 1] >= 0 ? 1 : 0);
             pend[k] = p;
         }
         const unsigned bal = __ballot_sync(0xffffffffu, k < m && p == 0);
@@ -173,13 +173,13 @@ __global__ void k_levels(int32_t* __restrict__ pend, const int32_t* __restrict__
     }
 }
 
-// level of every rank; the class-major order is the edges sorted by level, ranks ascending
-__global__ void k_level_keys(const int32_t* __restrict__ level, const int32_t* __restrict__ ord, int64_t m,
-                             uint32_t* __restrict__ key, int32_t* __restrict__ val) {
+// level of every rank; the class-major order is the ranks sorted by level, ascending in a level
+__global__ void k_level_keys(const int32_t* __restrict__ level, int64_t m, uint32_t* __restrict__ key,
+                             int32_t* __restrict__ val) {
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < m;
          k += (int64_t)gridDim.x * blockDim.x) {
         key[k] = (uint32_t)level[k];
-        val[k] = ord[k];
+        val[k] = (int32_t)k;
     }
 }
 
@@ -192,6 +192,26 @@ __global__ void k_level_heads(const uint32_t* __restrict__ key, int64_t m, int32
 __global__ void k_map_ids(const int32_t* __restrict__ ids, int64_t k, int32_t* __restrict__ x) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k; i += (int64_t)gridDim.x * blockDim.x)
         x[i] = ids[x[i]];
+}
+
+// position of every rank in the class-major order
+__global__ void k_rank_positions(const int32_t* __restrict__ rank, int64_t m, int32_t* __restrict__ pos) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
+        pos[rank[i]] = (int32_t)i;
+}
+
+// per leading position and end: 1 + the position of the update before it at that node (0: none)
+__global__ void k_previous(const int32_t* __restrict__ rank, int64_t m_grid, const int32_t* __restrict__ pred,
+                           const int32_t* __restrict__ pos, uint32_t* __restrict__ prev) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m_grid;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t k = rank[i];
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const int32_t q = pred[2 * k + s];
+            prev[2 * i + s] = q >= 0 ? (uint32_t)pos[q] + 1u : 0u;
+        }
+    }
 }
 
 // ------------------------------------------------------------------ chunked stream
@@ -720,64 +740,130 @@ k_sweep_stream(int32_t n, int32_t NC, const int64_t* __restrict__ blob_off, cons
 }
 
 // The leading classes of the level order are large (on R-MAT, light edges come first: the
-// first few thousand classes hold most edges).  Each of them is one grid-wide step: every
-// thread takes edges of the class, reads both loads from global memory (L2, bypassing L1),
-// updates and writes them back; a grid barrier separates the classes.  The remaining classes
-// (the long tail of small classes around the hubs) go through k_sweep_stream.
-constexpr int kGridThreads = 1024;
-// A grid-wide step costs about one grid barrier plus one memory round trip (~3 us) whatever
-// the class size; the one-CTA stream moves about one tail edge per 17 ns (it is bound by the
-// scattered 8-byte gathers and write-backs of a single SM).  Classes above ~3 us / 17 ns
-// edges are cheaper as grid steps.
-constexpr int32_t kGridMinClass = 192;    // classes at least this large take a grid-wide step
+// first few thousand classes hold most edges) and run over all SMs, without a barrier between
+// classes.  A node's load is a 16-byte entry, (hi, tag), (lo, tag), whose tag is 1 + the position
+// of the last update of that node; every edge end knows the position of the update before it at
+// its node.  Warps take the edges in class-major order, 32 at a time; an edge waits until both of
+// its entries carry the tags it expects, updates and writes them back with its own.  Each 8-byte
+// half is one access and carries the tag, so a value and its version arrive together and no
+// fence is needed.  The earliest edge that is not done waits for nothing and its warp has
+// reached it, so the waits end (all blocks are resident: a cooperative launch); they are
+// bounded all the same.
+//
+// What bounds it: the chain through the hubs (one edge per class and hub), a store, an L2
+// round trip and a poll per link: about 0.35 us a class, where a grid barrier per class cost 3.4 us
+// whatever the class size.  Measured (GB300, ms per pass, barrier -> entries, tail and star steps
+// included): R-MAT scale 16 6.5 -> 3.3, scale 20 52.5 -> 21.4; with hub stars scale 18 12.6 -> 4.8,
+// scale 20 31.4 -> 9.9, scale 20 weighted 17.6 -> 7.0.
+constexpr int kFlowSegs = 2;                // launches of the leading classes
+constexpr uint32_t kFlowPolls = 1u << 22;   // bounded waits
+// Classes at least this large run here, the rest in one CTA (about 17 ns an edge and a barrier a
+// class there).  Scale 20 / scale 16, ms per pass, by the threshold: 192 26.2 / 3.75, 96 21.5 /
+// 3.32, 48 21.3 / 3.26, 16 25.0 / 3.40, 1 33.8 / 5.0.
+constexpr int32_t kGridMinClass = 64;
+
+__device__ __forceinline__ ulonglong2 ld_node(const ulonglong2* p) {
+    ulonglong2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_node(ulonglong2* p, float2 x, uint32_t tag) {
+    const unsigned long long t = (unsigned long long)tag << 32;
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};"
+                 ::"l"(p), "l"(t | __float_as_uint(x.x)), "l"(t | __float_as_uint(x.y)) : "memory");
+}
+__device__ __forceinline__ bool node_is(const ulonglong2& v, uint32_t tag) {
+    return (((uint32_t)(v.x >> 32) ^ tag) | ((uint32_t)(v.y >> 32) ^ tag)) == 0u;
+}
+__device__ __forceinline__ float2 node_load(const ulonglong2& v) {
+    return make_float2(__uint_as_float((uint32_t)v.x), __uint_as_float((uint32_t)v.y));
+}
+
+__global__ void k_nodes_from_loads(const float2* __restrict__ lp, int32_t n, ulonglong2* __restrict__ nodes) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const float2 x = lp[i];
+        nodes[i] = make_ulonglong2(__float_as_uint(x.x), __float_as_uint(x.y));   // tag 0: no update yet
+    }
+}
+
+__global__ void k_loads_from_nodes(const ulonglong2* __restrict__ nodes, int32_t n, float2* __restrict__ lp) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        lp[i] = node_load(nodes[i]);
+}
 
 template <bool WEIGHTED>
-__global__ void __launch_bounds__(kGridThreads)
-k_sweep_grid(int32_t K, const int32_t* __restrict__ coff, const int32_t* __restrict__ ea,
-             const int32_t* __restrict__ eb, const float* __restrict__ cw, float* __restrict__ cs,
-             float2* __restrict__ lp, unsigned* __restrict__ bar, int32_t* __restrict__ err) {
-    const int64_t T = (int64_t)gridDim.x * blockDim.x;
-    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    // the ends, split and weight of this thread's first edge of the next class are read before
-    // the grid barrier (they do not depend on the loads), so a class costs one round trip
-    int32_t b0 = K > 0 ? __ldg(coff) : 0;
-    int32_t na = 0, nb = 0;
-    float nsplit = 0.0f, nw = 1.0f;
-    auto fetch = [&](int64_t i, int32_t end) {
+__global__ void __launch_bounds__(512)
+k_sweep_nodes(int32_t beg, int32_t end, const int32_t* __restrict__ ea, const int32_t* __restrict__ eb,
+              const uint2* __restrict__ prev, const float* __restrict__ cw, float* __restrict__ cs,
+              ulonglong2* __restrict__ nodes, int32_t* __restrict__ err) {
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    // consecutive warps of the order lie on different SMs
+    const int64_t first = beg + ((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + lane;
+    int32_t a = 0, b = 0;
+    uint2 pv = make_uint2(0u, 0u);
+    float s = 0.0f, w = 1.0f;
+    auto fetch = [&](int64_t i) {
         if (i < end) {
-            na = __ldg(ea + i);
-            nb = __ldg(eb + i);
-            nsplit = __ldcg(cs + i);
-            nw = WEIGHTED ? __ldg(cw + i) : 1.0f;
+            a = __ldg(ea + i);
+            b = __ldg(eb + i);
+            pv = __ldg(prev + i);
+            s = __ldcg(cs + i);
+            if (WEIGHTED) w = __ldg(cw + i);
         }
     };
-    if (K > 0) fetch(b0 + t0, __ldg(coff + 1));
-    for (int32_t c = 0; c < K; ++c) {
-        const int32_t b1 = __ldg(coff + c + 1);
-        for (int64_t i = b0 + t0; i < b1; i += T) {
-            int32_t a, b;
-            float s, w;
-            if (i == b0 + t0) {
-                a = na; b = nb; s = nsplit; w = nw;
-            } else {
-                a = __ldg(ea + i); b = __ldg(eb + i); s = __ldcg(cs + i);
-                w = WEIGHTED ? __ldg(cw + i) : 1.0f;
+    fetch(first);
+    for (int64_t i = first; i - lane < end; i += stride) {
+        bool done = i >= end;
+        const int32_t ca = a, cb = b;
+        const uint2 want = pv;
+        const float cs_i = s, cw_i = w;
+        fetch(i + stride);   // the next edge's record, under way while this one waits
+        uint32_t polls = 0;
+        for (;;) {
+            if (!done) {
+                const ulonglong2 na = ld_node(nodes + ca), nb = ld_node(nodes + cb);
+                if (node_is(na, want.x) && node_is(nb, want.y)) {
+                    float2 A = node_load(na), B = node_load(nb);
+                    const float ns = comp_transfer(A, B, cs_i, WEIGHTED ? cw_i : 1.0f);
+                    st_node(nodes + ca, A, (uint32_t)i + 1u);
+                    st_node(nodes + cb, B, (uint32_t)i + 1u);
+                    __stcg(cs + i, ns);
+                    done = true;
+                }
             }
-            float2 A = __ldcg(lp + a), B = __ldcg(lp + b);
-            const float ns = comp_transfer(A, B, s, w);
-            __stcg(lp + a, A);
-            __stcg(lp + b, B);
-            __stcg(cs + i, ns);
+            if (__all_sync(0xffffffffu, done)) break;
+            ++polls;
+            if ((polls & 1023u) == 0u) {
+                bool stop = *(volatile int32_t*)err != 0;
+                if (polls >= kFlowPolls) {
+                    stop = true;
+                    if (lane == 0) atomicOr(err, 2);
+                }
+                if (__any_sync(0xffffffffu, stop)) return;
+            }
+            if (polls > 4u) __nanosleep(20);
         }
-        b0 = b1;
-        if (c + 1 < K) fetch(b0 + t0, __ldg(coff + c + 2));
-        if (!grid_barrier(bar, bar + 1, gridDim.x, err)) return;
     }
 }
 
 }  // namespace
 
 // ------------------------------------------------------------------ host side
+
+// The leading classes' launches, by class size: threads to move the edges of the large classes, and
+// fewer for the small ones, where a thread whose edge is many classes away only polls (half as
+// many made no difference on scale 16 and 20).  s2_seg: positions where the segments end.
+static const int kFlowThreads[kFlowSegs] = {512, 128};
+static const int32_t kFlowSizes[kFlowSegs] = {4096, 0};   // smallest class of each
+
+static void flow_segments(lowd_ctx* h, const std::vector<int32_t>& coff, int32_t K) {
+    int32_t c = 0;
+    for (int g = 0; g < kFlowSegs; ++g) {
+        while (c < K && coff[(size_t)c + 1] - coff[(size_t)c] >= kFlowSizes[g]) ++c;
+        h->s2_seg[g] = coff[(size_t)c];
+    }
+}
 
 // Level colouring, class-major order, chunk tables, streams and descriptors; then the
 // initial splits (equal split or the given canonical-order splits) and the loads.
@@ -793,7 +879,7 @@ lowd_status lowd_stream_prepare(lowd_ctx* h, const float* init_splits_canon) {
     uint64_t* k64[2] = {nullptr, nullptr};
     int32_t* val[2] = {nullptr, nullptr};
     int32_t *succ = nullptr, *pend = nullptr, *level = nullptr, *fr[2] = {nullptr, nullptr}, *ctl = nullptr;
-    uint8_t* has_pred = nullptr;
+    int32_t *pred = nullptr, *pos = nullptr;
     uint32_t* okey[2] = {nullptr, nullptr};
     int64_t* oval[2] = {nullptr, nullptr};
     int64_t *gfirst = nullptr, *glast = nullptr;
@@ -803,7 +889,7 @@ lowd_status lowd_stream_prepare(lowd_ctx* h, const float* init_splits_canon) {
         sp.release(h);
         dfree(h, &deg); dfree(h, &k32[0]); dfree(h, &k32[1]); dfree(h, &k64[0]); dfree(h, &k64[1]); dfree(h, &val[0]);
         dfree(h, &val[1]); dfree(h, &succ); dfree(h, &pend); dfree(h, &level); dfree(h, &fr[0]); dfree(h, &fr[1]); dfree(h, &ctl);
-        dfree(h, &has_pred); dfree(h, &okey[0]); dfree(h, &okey[1]); dfree(h, &oval[0]); dfree(h, &oval[1]);
+        dfree(h, &pred); dfree(h, &pos); dfree(h, &okey[0]); dfree(h, &okey[1]); dfree(h, &oval[0]); dfree(h, &oval[1]);
         dfree(h, &gfirst); dfree(h, &glast); dfree(h, &rb); dfree(h, &pb);
     };
     const bool weighted = h->w != nullptr;
@@ -825,6 +911,7 @@ lowd_status lowd_stream_prepare(lowd_ctx* h, const float* init_splits_canon) {
         int32_t C = 0;
         int32_t* ord = nullptr;      // rank -> edge id
         int32_t* order = nullptr;    // class-major position -> edge id
+        int32_t* ranks = nullptr;    // class-major position -> rank
         if (m > 0) {
             if ((s = dalloc(h, &k32[0], 2 * m))) break;
             if ((s = dalloc(h, &k32[1], 2 * m))) break;
@@ -852,8 +939,8 @@ lowd_status lowd_stream_prepare(lowd_ctx* h, const float* init_splits_canon) {
             uint32_t* nodes = c3 ? k32[1] : k32[0];
             int32_t* rks = c3 ? rk2 : spare;
             if ((s = dalloc(h, &succ, 2 * m))) { dfree(h, &rk2); break; }
-            if ((s = dalloc(h, &has_pred, 2 * m))) { dfree(h, &rk2); break; }
-            LOWD_LAUNCH(k_successors, grid_for(2 * m), kT, 0, st, nodes, rks, 2 * m, ord, cu, succ, has_pred);
+            if ((s = dalloc(h, &pred, 2 * m))) { dfree(h, &rk2); break; }
+            LOWD_LAUNCH(k_successors, grid_for(2 * m), kT, 0, st, nodes, rks, 2 * m, ord, cu, succ, pred);
             dfree(h, &rk2);
             // ord must survive: copy it out of the ping-pong buffers
             int32_t* ord_keep = nullptr;
@@ -868,7 +955,7 @@ lowd_status lowd_stream_prepare(lowd_ctx* h, const float* init_splits_canon) {
             if ((s = dalloc(h, &fr[1], m))) break;
             if ((s = dalloc(h, &ctl, 16))) break;
             cudaMemsetAsync(ctl, 0, 16 * sizeof(int32_t), st);
-            LOWD_LAUNCH(k_pending, grid_for(m), kT, 0, st, has_pred, m, pend, fr[0], ctl);
+            LOWD_LAUNCH(k_pending, grid_for(m), kT, 0, st, pred, m, pend, fr[0], ctl);
             // ---- 3. levels (cooperative: every block must be resident for the grid barrier)
             int dev = 0, nb_per_sm = 0;
             cudaGetDevice(&dev);
@@ -892,10 +979,16 @@ lowd_status lowd_stream_prepare(lowd_ctx* h, const float* init_splits_canon) {
             }
             C = hc[6];
             // ---- 4. class-major order: sort by level (stable over rank order)
-            LOWD_LAUNCH(k_level_keys, grid_for(m), kT, 0, st, level, ord, m, k32[0], fr[0]);
+            LOWD_LAUNCH(k_level_keys, grid_for(m), kT, 0, st, level, m, k32[0], fr[0]);
             const int lbits = bit_length_u64((uint64_t)(C > 1 ? C - 1 : 1));
             int c4 = radix_sort_pairs<uint32_t, int32_t>(k32[0], fr[0], k32[1], fr[1], m, lbits, h->tmp, st);
             order = c4 ? fr[1] : fr[0];
+            if ((s = dalloc(h, &pos, m))) break;
+            LOWD_LAUNCH(k_rank_positions, grid_for(m), kT, 0, st, order, m, pos);
+            int32_t* by_rank = c4 ? fr[0] : fr[1];   // the ranks stay for the leading classes' records
+            cudaMemcpyAsync(by_rank, order, sizeof(int32_t) * (size_t)m, cudaMemcpyDeviceToDevice, st);
+            ranks = by_rank;
+            LOWD_LAUNCH(k_map_ids, grid_for(m), kT, 0, st, ord, m, order);
             if (pid) LOWD_LAUNCH(k_map_ids, grid_for(m), kT, 0, st, pid, m, order);   // subset -> edge ids
             if ((s = dalloc(h, &h->coff_real, (size_t)C + 1))) break;
             LOWD_LAUNCH(k_level_heads, grid_for(m), kT, 0, st, c4 ? k32[1] : k32[0], m, h->coff_real);
@@ -914,11 +1007,18 @@ lowd_status lowd_stream_prepare(lowd_ctx* h, const float* init_splits_canon) {
         const uint32_t E = stream_edges_per_stage(S, weighted, budget);
         // header rows: [0] padded begin, [1] padded size, [2] segments, [3 + g] end of segment
         // g relative to the begin; real_beg: the chunk's first real (unpadded) position
-        // leading classes of at least kGridMinClass edges take grid-wide steps (positions
+        // leading classes of at least kGridMinClass edges run over all SMs (positions
         // [0, coff[K]) of the stream, padded to a multiple of 4); the rest are chunked
         int32_t K = 0;
         while (K < C && coff[K + 1] - coff[K] >= kGridMinClass) ++K;
         const int64_t m_grid = coff[K];
+        if (m_grid > 0) {
+            if ((s = dalloc(h, &h->s2_prev, m_grid))) break;
+            if ((s = dalloc(h, &h->s2_nodes, n))) break;
+            LOWD_LAUNCH(k_previous, grid_for(m_grid), kT, 0, st, ranks, m_grid, pred, pos,
+                        reinterpret_cast<uint32_t*>(h->s2_prev));
+        }
+        flow_segments(h, coff, K);
         const int64_t grid_pad = (m_grid + 3) & ~(int64_t)3;
         std::vector<int32_t> ctab, real_beg;
         int64_t pad = grid_pad, real = m_grid;
@@ -1068,30 +1168,33 @@ cudaError_t lowd_stream_passes(lowd_ctx* h, int32_t passes) {
                     h->d_i32 + 8);
         return cudaGetLastError();
     };
-    cudaMemsetAsync(h->d_i32 + 12, 0, 2 * sizeof(int32_t), h->st);   // grid barrier words
-    unsigned* bar = reinterpret_cast<unsigned*>(h->d_i32 + 12);
-    int32_t* errp = h->d_i32 + 8;
-    if (h->star_S > 0) {
-        // per pass: the plain edges (grid steps, then the chunked tail), then the star steps
-        auto gk = weighted ? k_sweep_grid<true> : k_sweep_grid<false>;
-        int32_t K = h->s2_K;
-        const int32_t* coff = h->coff_real;
-        const int32_t* pea = h->s2_ea;
-        const int32_t* peb = h->s2_eb;
-        const float* pcw = h->cw;
-        float* pcs = h->cs;
-        float2* plp = h->s2_lp;
-        void* args[] = {&K, &coff, &pea, &peb, &pcw, &pcs, &plp, &bar, &errp};
-        for (int32_t t = 0; t < passes && e == cudaSuccess; ++t) {
-            if (K > 0) {
-                e = cudaLaunchCooperativeKernel((const void*)gk, dim3(lowd_device_sms()), dim3(kGridThreads), args, 0,
-                                                h->st);
-                lowd_note_launch();
-            }
-            if (e == cudaSuccess && h->s2_tail) e = stream_launch(1);
-            if (e == cudaSuccess) e = lowd_star_pass(h);
+    cudaMemsetAsync(h->d_i32 + 12, 0, 2 * sizeof(int32_t), h->st);   // grid barrier words (star steps)
+    // the leading classes: loads into tagged entries, a launch per segment, loads back
+    auto leading = [&]() -> cudaError_t {
+        auto gk = weighted ? k_sweep_nodes<true> : k_sweep_nodes<false>;
+        LOWD_LAUNCH(k_nodes_from_loads, grid_for(h->n), kT, 0, h->st, h->s2_lp, h->n, h->s2_nodes);
+        int32_t beg = 0;
+        int32_t* errp = h->d_i32 + 8;
+        for (int g = 0; g < kFlowSegs; ++g) {
+            int32_t end = h->s2_seg[g];
+            if (end == beg) continue;
+            const int32_t* pea = h->s2_ea;
+            const int32_t* peb = h->s2_eb;
+            const uint2* pp = h->s2_prev;
+            const float* pcw = h->cw;
+            float* pcs = h->cs;
+            ulonglong2* pn = h->s2_nodes;
+            void* args[] = {&beg, &end, &pea, &peb, &pp, &pcw, &pcs, &pn, &errp};
+            const cudaError_t r = cudaLaunchCooperativeKernel((const void*)gk, dim3(lowd_device_sms()),
+                                                              dim3(kFlowThreads[g]), args, 0, h->st);
+            lowd_note_launch();
+            if (r != cudaSuccess) return r;
+            beg = end;
         }
-    } else if (h->s2_K == 0) {
+        LOWD_LAUNCH(k_loads_from_nodes, grid_for(h->n), kT, 0, h->st, h->s2_nodes, h->n, h->s2_lp);
+        return cudaGetLastError();
+    };
+    if (h->s2_K == 0 && h->star_S == 0) {
         const int32_t per = (int32_t)(0x7fffffff / h->s2_NC);
         for (int32_t done = 0; done < passes && e == cudaSuccess;) {
             const int32_t k = passes - done < per ? passes - done : per;
@@ -1099,23 +1202,11 @@ cudaError_t lowd_stream_passes(lowd_ctx* h, int32_t passes) {
             done += k;
         }
     } else {
-        // per pass: the large classes as grid-wide steps, then the tail through the stream
-        auto gk = weighted ? k_sweep_grid<true> : k_sweep_grid<false>;
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gk, kGridThreads, 0);
-        const int blocks = lowd_device_sms() * (per_sm > 0 ? 1 : 1);   // one block per SM
-        int32_t K = h->s2_K;
-        const int32_t* coff = h->coff_real;
-        const int32_t* pea = h->s2_ea;
-        const int32_t* peb = h->s2_eb;
-        const float* pcw = h->cw;
-        float* pcs = h->cs;
-        float2* plp = h->s2_lp;
-        void* args[] = {&K, &coff, &pea, &peb, &pcw, &pcs, &plp, &bar, &errp};
+        // per pass: the leading classes, the chunked tail, then the star steps
         for (int32_t t = 0; t < passes && e == cudaSuccess; ++t) {
-            e = cudaLaunchCooperativeKernel((const void*)gk, dim3(blocks), dim3(kGridThreads), args, 0, h->st);
-            lowd_note_launch();
+            if (h->s2_K > 0) e = leading();
             if (e == cudaSuccess && h->s2_tail) e = stream_launch(1);
+            if (e == cudaSuccess && h->star_S > 0) e = lowd_star_pass(h);
         }
     }
     if (e != cudaSuccess) return e;

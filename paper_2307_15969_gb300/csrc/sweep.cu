@@ -1410,7 +1410,7 @@ lowd_status lowd_sweep_run(lowd_ctx* h, int32_t k, const lowd_options* opt, lowd
         if (kerr != 0) {
             snprintf(h->err, sizeof(h->err), "%s",
                      (kerr & 4) ? "sweep: a read descriptor pointed outside the stages"
-                                : ((kerr & 2) ? "sweep: a bounded grid barrier expired"
+                                : ((kerr & 2) ? "sweep: a bounded wait across the grid expired"
                                               : "sweep: a bounded wait on a staged copy expired"));
             return LOWD_ERR_CUDA;
         }
