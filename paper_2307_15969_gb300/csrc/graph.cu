@@ -10,6 +10,7 @@
 //    renumbered by ascending original id and its edges in their original order.
 #include "ctx.cuh"
 #include "prims.cuh"
+#include "async.cuh"
 
 using namespace lowd;
 
@@ -263,28 +264,28 @@ __device__ __forceinline__ bool below_bound(unsigned long long d, int64_t N, int
     return lhs < (unsigned __int128)(uint64_t)W;
 }
 
-// Round r of Algorithm 2, node side: among the listed live nodes, mark every node whose
-// current degree is below the density bound (its removal round, and its bit in the removed
-// set); count them.  keep[i] = 1 for survivors.  Node ids are those of the current id space:
-// orig maps them to the input's ids (null: the same ids).
-__global__ void k_prune_mark(const int32_t* __restrict__ act, int64_t nact,
-                             const unsigned long long* __restrict__ deg, int64_t N, int64_t W,
-                             int32_t r, const int32_t* __restrict__ orig, int32_t* __restrict__ rr,
-                             uint32_t* __restrict__ dead, int32_t* __restrict__ keep,
-                             unsigned long long* __restrict__ removed) {
+// A round of Algorithm 2, node side: among the live nodes, mark every node whose current degree is
+// below the density bound (its removal round, and its bit in the removed set); returns how many
+// this thread marked.  Node ids are those of the current id space of n1 nodes: orig maps them to
+// the input's ids (null: the same ids).
+__device__ __forceinline__ unsigned long long prune_mark(int64_t n1, const unsigned long long* deg, int64_t N, int64_t W,
+                                                         int32_t r, const int32_t* orig, int32_t* rr, uint32_t* dead) {
     unsigned long long c = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nact;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t x = act[i];
-        bool rem = below_bound(deg[x], N, W);
-        if (rem) {
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n1; x += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t bit = 1u << (x & 31);
+        // (a bit set in this round is another node's: this thread alone sets x's)
+        if (!(__ldcg(dead + (x >> 5)) & bit) && below_bound(__ldcg(deg + x), N, W)) {
             rr[orig ? orig[x] : x] = r;
-            atomicOr(&dead[x >> 5], 1u << (x & 31));
+            atomicOr(&dead[x >> 5], bit);
             ++c;
         }
-        keep[i] = rem ? 0 : 1;
     }
-    c = warp_sum(c);
+    return c;
+}
+
+__global__ void k_prune_mark(int64_t n, const unsigned long long* __restrict__ deg, int64_t W, int32_t* __restrict__ rr,
+                             uint32_t* __restrict__ dead, unsigned long long* __restrict__ removed) {
+    const unsigned long long c = warp_sum(prune_mark(n, deg, n, W, 1, nullptr, rr, dead));
     if (lane_id() == 0 && c) atomicAdd(removed, c);
 }
 
@@ -313,16 +314,13 @@ __device__ __forceinline__ int32_t rank_of(uint2 p, int32_t x) {
     return (int32_t)(p.y + (uint32_t)__popc(~p.x & ((1u << (x & 31)) - 1u)));
 }
 
+// (The later rounds run in one kernel: their lists and removed set change between rounds, so they
+// are read by plain loads, not through the non-coherent path.)
 template <bool RELABEL>
-__global__ void __launch_bounds__(kT, 4)
-k_prune_edges(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
-              const int64_t* __restrict__ ew, int64_t me, const uint32_t* __restrict__ dead,
-              const uint2* __restrict__ rank_words, const unsigned long long* __restrict__ removed,
-              unsigned long long* __restrict__ deg,
-              unsigned long long* __restrict__ removedW,
-              int32_t* __restrict__ nu, int32_t* __restrict__ nv,
-              int64_t* __restrict__ nw, unsigned long long* __restrict__ ncount) {
-    if (*removed == 0) return;   // the same value for every thread: no barrier is skipped
+__device__ __forceinline__ void prune_edges(const int32_t* eu, const int32_t* ev, const int64_t* ew, int64_t me,
+                                            const uint32_t* dead, const uint2* rank_words, unsigned long long* deg,
+                                            unsigned long long* removedW, int32_t* nu, int32_t* nv, int64_t* nw,
+                                            unsigned long long* ncount) {
     __shared__ unsigned long long sh_base;
     __shared__ int32_t sh_warp[kT / 32];
     const unsigned lane = lane_id();
@@ -362,8 +360,8 @@ k_prune_edges(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
                 na = rank_of(pa, a[i]);
                 nb = rank_of(pb, b[i]);
             } else {
-                ra = ok && ((__ldg(dead + (a[i] >> 5)) >> (a[i] & 31)) & 1u);
-                rb = ok && ((__ldg(dead + (b[i] >> 5)) >> (b[i] & 31)) & 1u);
+                ra = ok && ((dead[a[i] >> 5] >> (a[i] & 31)) & 1u);
+                rb = ok && ((dead[b[i] >> 5] >> (b[i] & 31)) & 1u);
             }
             if (ra || rb) acc += (unsigned long long)x[i];
             const int32_t da = (ok && rb && !ra) ? a[i] : -1;   // surviving end of a removed edge
@@ -410,6 +408,71 @@ k_prune_edges(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
     if (lane_id() == 0 && acc) atomicAdd(removedW, acc);
 }
 
+// The first round's edges.
+__global__ void __launch_bounds__(kT, 4)
+k_prune_edges(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
+              const int64_t* __restrict__ ew, int64_t me, const uint2* __restrict__ rank_words,
+              const unsigned long long* __restrict__ removed, unsigned long long* __restrict__ deg,
+              unsigned long long* __restrict__ removedW, int32_t* __restrict__ nu, int32_t* __restrict__ nv,
+              int64_t* __restrict__ nw, unsigned long long* __restrict__ ncount) {
+    if (*removed == 0) return;   // the same value for every thread: no barrier is skipped
+    prune_edges<true>(eu, ev, ew, me, nullptr, rank_words, deg, removedW, nu, nv, nw, ncount);
+}
+
+// The rounds after the first, in one cooperative launch: mark, a grid barrier, edges, a grid
+// barrier.  A round of its own launches and read-back costs about 60 us whatever its size: a
+// 2,000-node network takes 20 rounds.  ctl: [0..8] the counters (removed nodes, removed weight,
+// surviving edges) of the rounds r = 0, 1, 2 mod 3 (the first round's are in slot 1, the others
+// zero), [9] live nodes, [10] live edges and [11] rounds on return.  The lists change places every
+// round; a round that removes nothing leaves them.
+struct PruneRounds {
+    int64_t n, m, W;             // the input's nodes and edges, and its weight
+    const int32_t* orig;
+    int32_t* rr;
+    uint32_t* dead;
+    unsigned long long* deg;
+    int32_t* eu[2];              // the live edges after the first round are in [0]
+    int32_t* ev[2];
+    int64_t* ew[2];
+    unsigned long long* ctl;
+    unsigned* bar;
+    int32_t* err;
+};
+
+__global__ void __launch_bounds__(kT, 4) k_prune_rounds(const PruneRounds p) {
+    volatile unsigned long long* c = p.ctl;
+    int64_t N = p.n - (int64_t)c[3], W = p.W - (int64_t)c[4], me = (int64_t)c[5];
+    const int64_t n1 = N;        // the id space of the first round's survivors
+    const bool any = c[3] != 0;
+    if (!any) me = p.m;
+    int32_t r = any ? 1 : 0;
+    bool odd = false;            // which lists hold the live edges
+    while (any && N > 0) {
+        unsigned long long* slot = p.ctl + 3 * ((r + 1) % 3);
+        // the slot of the round after this one, last read two rounds ago
+        if (blockIdx.x == 0 && threadIdx.x < 3) p.ctl[3 * ((r + 2) % 3) + threadIdx.x] = 0;
+        const unsigned long long k = warp_sum(prune_mark(n1, p.deg, N, W, r + 1, p.orig, p.rr, p.dead));
+        if (lane_id() == 0 && k) atomicAdd(&slot[0], k);
+        if (!grid_barrier(p.bar, p.bar + 1, gridDim.x, p.err)) return;
+        const int64_t gone = (int64_t)*(volatile unsigned long long*)&slot[0];
+        if (gone == 0) break;
+        prune_edges<false>(odd ? p.eu[1] : p.eu[0], odd ? p.ev[1] : p.ev[0], odd ? p.ew[1] : p.ew[0], me, p.dead, nullptr,
+                           p.deg, &slot[1], odd ? p.eu[0] : p.eu[1], odd ? p.ev[0] : p.ev[1], odd ? p.ew[0] : p.ew[1],
+                           &slot[2]);
+        if (!grid_barrier(p.bar, p.bar + 1, gridDim.x, p.err)) return;
+        N -= gone;
+        W -= (int64_t)*(volatile unsigned long long*)&slot[1];
+        me = (int64_t)*(volatile unsigned long long*)&slot[2];
+        odd = !odd;
+        ++r;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        p.ctl[9] = (unsigned long long)N;
+        p.ctl[10] = (unsigned long long)me;
+        p.ctl[11] = (unsigned long long)r;
+    }
+}
+
 // Rank words of the first round's renumbering: surviving ids per word of the removed set
 // (ids past the last node count too, but only the words before a word enter its rank), then,
 // after their exclusive scan, each word with the survivors before it.
@@ -442,18 +505,6 @@ __global__ void k_relabel_nodes(const uint2* __restrict__ rw, int32_t n,
     }
 }
 
-// Stable compaction of the live node list by flag, survivors renumbered by their rank words.
-__global__ void k_compact_ranked(const int32_t* __restrict__ act, const int32_t* __restrict__ flag,
-                                 const int32_t* __restrict__ pos, int64_t n, const uint2* __restrict__ rw,
-                                 int32_t* __restrict__ out) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        if (flag[i]) {
-            const int32_t x = act[i];
-            out[pos[i]] = rank_of(rw[x >> 5], x);
-        }
-}
-
 // The removed set over the input's ids, from the removal rounds (one warp per word).
 __global__ void k_dead_from_rounds(const int32_t* __restrict__ rr, int32_t n, uint32_t* __restrict__ dead) {
     const int64_t words = ((int64_t)n + 31) / 32;
@@ -463,14 +514,6 @@ __global__ void k_dead_from_rounds(const int32_t* __restrict__ rr, int32_t n, ui
         const unsigned bits = __ballot_sync(0xffffffffu, x < n && rr[x] >= 0);
         if (lane_id() == 0) dead[w] = bits;
     }
-}
-
-template <class T>
-__global__ void k_compact_by_flag(const T* __restrict__ in, const int32_t* __restrict__ flag,
-                                  const int32_t* __restrict__ pos, int64_t n, T* __restrict__ out) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        if (flag[i]) out[pos[i]] = in[i];
 }
 
 __global__ void k_keep_nodes(const int32_t* __restrict__ rr, int32_t n, int32_t* __restrict__ keep) {
@@ -707,24 +750,24 @@ lowd_status lowd_graph_prune(lowd_ctx* h, int32_t* rounds_out) {
     unsigned long long* deg = nullptr;
     uint64_t* dkey[2] = {nullptr, nullptr};
     int32_t* dval[2] = {nullptr, nullptr};
-    int32_t *act = nullptr, *act2 = nullptr, *keep = nullptr, *pos = nullptr;
+    int32_t *keep = nullptr, *pos = nullptr;
     int32_t *eu[2] = {nullptr, nullptr}, *ev[2] = {nullptr, nullptr};
     int64_t* ew[2] = {nullptr, nullptr};
     int32_t *keepe = nullptr, *epos = nullptr, *nmap = nullptr;
     uint32_t* dead = nullptr;   // nodes removed so far, one bit each
     uint2* rw = nullptr;        // rank words of the first round's renumbering
     int32_t *wcnt = nullptr, *wpre = nullptr, *orig = nullptr;
-    unsigned long long* deg2 = nullptr;
+    unsigned long long *deg2 = nullptr, *ctl = nullptr;
     int32_t *nu = nullptr, *nv = nullptr;
     float* nw = nullptr;
     int64_t* nwu = nullptr;
     lowd_status s = LOWD_OK;
     auto cleanup = [&]() {
         dfree(h, &deg); dfree(h, &dkey[0]); dfree(h, &dkey[1]); dfree(h, &dval[0]); dfree(h, &dval[1]);
-        dfree(h, &act); dfree(h, &act2); dfree(h, &keep); dfree(h, &pos);
+        dfree(h, &keep); dfree(h, &pos);
         dfree(h, &eu[0]); dfree(h, &eu[1]); dfree(h, &ev[0]); dfree(h, &ev[1]); dfree(h, &ew[0]); dfree(h, &ew[1]);
         dfree(h, &keepe); dfree(h, &epos); dfree(h, &nmap); dfree(h, &dead); dfree(h, &nu); dfree(h, &nv); dfree(h, &nw); dfree(h, &nwu);
-        dfree(h, &rw); dfree(h, &wcnt); dfree(h, &wpre); dfree(h, &orig); dfree(h, &deg2);
+        dfree(h, &rw); dfree(h, &wcnt); dfree(h, &wpre); dfree(h, &orig); dfree(h, &deg2); dfree(h, &ctl);
     };
     do {
         if ((s = dalloc(h, &deg, n))) break;
@@ -765,87 +808,71 @@ lowd_status lowd_graph_prune(lowd_ctx* h, int32_t* rounds_out) {
         } else {
             W = m;
         }
-        int64_t N = n;
         if ((s = dalloc(h, &dead, ((size_t)n + 31) / 32))) break;
         cudaMemsetAsync(dead, 0, sizeof(uint32_t) * (((size_t)n + 31) / 32), st);
 
-        // live node list (degree order) and live edge list
-        if ((s = dalloc(h, &act, n))) break;
-        if ((s = dalloc(h, &act2, n))) break;
+        // ---- the first round: renumbers its survivors by rank (ascending ids)
         if ((s = dalloc(h, &keep, n))) break;
         if ((s = dalloc(h, &pos, n))) break;
-        cudaMemcpyAsync(act, h->sort_perm, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, st);
-        int64_t nact = n;
-        if ((s = dalloc(h, &eu[1], m))) break;
-        if ((s = dalloc(h, &ev[1], m))) break;
-        if (h->wu && (s = dalloc(h, &ew[1], m))) break;
-        const int32_t* cu_ = h->u;
-        const int32_t* cv_ = h->v;
-        const int64_t* cw_ = h->wu;
-        int64_t me = m;
-        int nxt = 1;
-        int32_t r = 0;
-        unsigned long long* removed = (unsigned long long*)(h->d_i64 + 4);
-        unsigned long long* removedW = (unsigned long long*)(h->d_i64 + 5);
-        unsigned long long* ncount = (unsigned long long*)(h->d_i64 + 6);
+        for (int i = 0; i < 2; ++i) {
+            if ((s = dalloc(h, &eu[i], m)) || (s = dalloc(h, &ev[i], m)) || (h->wu && (s = dalloc(h, &ew[i], m)))) break;
+        }
+        if (s) break;
         const int64_t Wn = ((int64_t)n + 31) / 32;   // words of the removed set over the input's ids
         if ((s = dalloc(h, &rw, Wn))) break;
         if ((s = dalloc(h, &wcnt, Wn))) break;
         if ((s = dalloc(h, &wpre, Wn))) break;
-        while (N > 0) {
-            int32_t rnext = r + 1;
-            const bool relabel = r == 0;   // the first round renumbers its survivors
-            cudaMemsetAsync(h->d_i64 + 4, 0, 3 * sizeof(int64_t), st);
-            LOWD_LAUNCH(k_prune_mark, grid_for(nact), kT, 0, st, act, nact, deg, N, W, rnext, orig, h->removal_round,
-                        dead, keep, removed);
-            if (relabel) {
-                LOWD_LAUNCH(k_word_alive, grid_for(Wn), kT, 0, st, dead, Wn, wcnt);
-                scan_exclusive<int32_t>(wcnt, wpre, Wn, nullptr, h->tmp, st);
-                LOWD_LAUNCH(k_rank_words, grid_for(Wn), kT, 0, st, dead, wpre, Wn, rw);
-            }
-            if (me > 0) {
-                const unsigned ge = lowd_grid_for(me, kPruneTile, 4);
-                if (relabel)
-                    LOWD_LAUNCH(k_prune_edges<true>, ge, kT, 0, st, cu_, cv_, cw_, me, dead, rw, removed, deg,
-                                removedW, eu[nxt], ev[nxt], ew[nxt], ncount);
-                else
-                    LOWD_LAUNCH(k_prune_edges<false>, ge, kT, 0, st, cu_, cv_, cw_, me, dead, rw, removed, deg,
-                                removedW, eu[nxt], ev[nxt], ew[nxt], ncount);
-            }
-            if (cudaGetLastError() != cudaSuccess) { s = h->fail(cudaGetLastError()); break; }
-            if (cudaMemcpyAsync(h->h_pin, h->d_i64 + 4, 3 * sizeof(int64_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-                cudaStreamSynchronize(st) != cudaSuccess) { s = h->fail(cudaGetLastError()); break; }
-            int64_t k = h->h_pin[0];
-            if (k == 0) break;  // the edge pass saw no removed end and kept every edge
-            r = rnext;
-            N -= k;
-            W -= h->h_pin[1];
-            cu_ = eu[nxt]; cv_ = ev[nxt]; cw_ = ew[nxt];
-            me = h->h_pin[2];
-            if (!eu[1 - nxt] && (s = dalloc(h, &eu[1 - nxt], m))) break;
-            if (!ev[1 - nxt] && (s = dalloc(h, &ev[1 - nxt], m))) break;
-            if (h->wu && !ew[1 - nxt] && (s = dalloc(h, &ew[1 - nxt], m))) break;
-            nxt = 1 - nxt;
-            // stable compaction of the live node list
-            scan_exclusive<int32_t>(keep, pos, nact, h->d_i32 + 3, h->tmp, st);
-            if (relabel) {
-                // the survivors' degrees, input ids and live list in the new id space (the edge
-                // list already carries the new ids); the removed set restarts there
-                if ((s = dalloc(h, &deg2, N))) break;
-                if ((s = dalloc(h, &orig, N))) break;
-                LOWD_LAUNCH(k_relabel_nodes, grid_for(n), kT, 0, st, rw, n, deg, deg2, orig);
-                dfree(h, &deg);
-                deg = deg2;
-                deg2 = nullptr;
-                LOWD_LAUNCH(k_compact_ranked, grid_for(nact), kT, 0, st, act, keep, pos, nact, rw, act2);
-                cudaMemsetAsync(dead, 0, sizeof(uint32_t) * (size_t)((N + 31) / 32), st);
-            } else {
-                LOWD_LAUNCH(k_compact_by_flag<int32_t>, grid_for(nact), kT, 0, st, act, keep, pos, nact, act2);
-            }
-            int32_t* t = act; act = act2; act2 = t;
-            nact = N;
+        if ((s = dalloc(h, &deg2, n))) break;
+        if ((s = dalloc(h, &orig, n))) break;
+        if ((s = dalloc(h, &ctl, 16))) break;
+        cudaMemsetAsync(ctl, 0, 16 * sizeof(unsigned long long), st);   // [14]: the barrier words, [15]: error
+        LOWD_LAUNCH(k_prune_mark, grid_for(n), kT, 0, st, (int64_t)n, deg, W, h->removal_round, dead, ctl + 3);
+        LOWD_LAUNCH(k_word_alive, grid_for(Wn), kT, 0, st, dead, Wn, wcnt);
+        scan_exclusive<int32_t>(wcnt, wpre, Wn, nullptr, h->tmp, st);
+        LOWD_LAUNCH(k_rank_words, grid_for(Wn), kT, 0, st, dead, wpre, Wn, rw);
+        if (m > 0)
+            LOWD_LAUNCH(k_prune_edges, lowd_grid_for(m, kPruneTile, 4), kT, 0, st, h->u, h->v, h->wu, m, rw, ctl + 3, deg,
+                        ctl + 4, eu[0], ev[0], ew[0], ctl + 5);
+        // the survivors' degrees and input ids in the new id space (the edge list already carries the
+        // new ids); the removed set restarts there
+        LOWD_LAUNCH(k_relabel_nodes, grid_for(n), kT, 0, st, rw, n, deg, deg2, orig);
+        cudaMemsetAsync(dead, 0, sizeof(uint32_t) * (size_t)Wn, st);
+        // ---- the other rounds, in one launch: as many blocks as the edges or nodes can use
+        int per_sm = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_prune_rounds, kT, 0);
+        int64_t blocks = (m + kPruneTile - 1) / kPruneTile;
+        if (blocks < ((int64_t)n + 4 * kT - 1) / (4 * kT)) blocks = ((int64_t)n + 4 * kT - 1) / (4 * kT);
+        const int64_t most = (int64_t)lowd_device_sms() * (per_sm < 4 ? (per_sm > 0 ? per_sm : 1) : 4);
+        if (blocks > most) blocks = most;
+        if (blocks < 1) blocks = 1;
+        PruneRounds pr;
+        pr.n = n;
+        pr.m = m;
+        pr.W = W;
+        pr.orig = orig;
+        pr.rr = h->removal_round;
+        pr.dead = dead;
+        pr.deg = deg2;
+        for (int i = 0; i < 2; ++i) { pr.eu[i] = eu[i]; pr.ev[i] = ev[i]; pr.ew[i] = ew[i]; }
+        pr.ctl = ctl;
+        pr.bar = reinterpret_cast<unsigned*>(ctl + 14);
+        pr.err = reinterpret_cast<int32_t*>(ctl + 15);
+        void* args[] = {&pr};
+        cudaError_t ce = cudaGetLastError();
+        if (ce == cudaSuccess)
+            ce = cudaLaunchCooperativeKernel((const void*)k_prune_rounds, dim3((unsigned)blocks), dim3(kT), args, 0, st);
+        lowd_note_launch();
+        if (ce == cudaSuccess)
+            ce = cudaMemcpyAsync(h->h_pin, ctl, 16 * sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+        if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+        if (ce != cudaSuccess) { s = h->fail(ce); break; }
+        if (*(int32_t*)(h->h_pin + 15) != 0) {
+            snprintf(h->err, sizeof(h->err), "prune: a bounded grid barrier expired");
+            s = LOWD_ERR_CUDA;
+            break;
         }
-        if (s) break;
+        const int64_t N = h->h_pin[9], me = h->h_pin[10];
+        const int32_t r = (int32_t)h->h_pin[11];
         h->prune_rounds = r;
         // the removed set over the input's ids, for the compaction to H
         LOWD_LAUNCH(k_dead_from_rounds, lowd_grid_for(Wn, kT / 32), kT, 0, st, h->removal_round, n, dead);
