@@ -45,8 +45,9 @@
 // critical path lie the steps at the diagonal and the right edge (150 to 190), a lag of about
 // three steps per tile, since inputs are checked four at a time, and the way between blocks.
 // Measured (GB300, per pass, against the one-CTA sweep of one barrier per class): n 9,109,
-// 6.25 M edges 1,130 us (was 2,705); n 9,110 1,807 us (2,705); n 4,047 488 us (701); n 6,193
-// weighted 756 us (1,189); n 307 29 us (111); n 71 7.9 us (22); G(4400, 0.95) 1,218 us (4,106).
+// 6.25 M edges 1,066 us (was 2,705); n 9,110 1,807 us (2,705); n 4,047 457 us (701); n 6,193
+// weighted 736 us (1,189); n 307 29 us (111); n 71 7.9 us (22);
+// G(4400, 0.95) 1,218 us (4,106).
 #include "ctx.cuh"
 #include "prims.cuh"
 #include "async.cuh"
@@ -60,7 +61,8 @@ namespace {
 constexpr int kT = 256;
 inline unsigned grid_for(int64_t n) { return lowd_grid_for(n, kT); }
 
-constexpr int kPairs = 4;             // pairs of tiles per block (two warps per scheduler)
+constexpr int kPairs = 4;             // most pairs of tiles per block of several (two warps per scheduler)
+constexpr int kPairsOdd = 2;          // odd n, while the SMs hold a block each
 constexpr int kMaxW = 5;              // the most, in a block alone
 constexpr int kPad = 96;              // steps of a lap beyond P: drained lanes, read-ahead, tags
 constexpr size_t kSmemMost = 226 * 1024;   // dynamic shared memory of a block (227 KB less the static part)
@@ -1034,7 +1036,7 @@ lowd_status lowd_sys_class_sizes(lowd_ctx* h, const int32_t* u, const int32_t* v
 // Whether the array serves this graph of C classes.  Its cells grow with n^2, so they are bounded
 // by 2^26 (268 MB: n up to about 11,500 whatever the density) or 16 cells per edge; sparser
 // graphs keep the staged sweep, whose memory grows with the edges.  Measured per class: the array
-// takes 88 (n 129) to 124 ns (n 9,109) for odd n, the one-CTA kernels 148 ns (60 edges a class) to
+// takes 88 (n 129) to 117 ns (n 9,109) for odd n, the one-CTA kernels 148 ns (60 edges a class) to
 // 297 (710) and 933 (2,090), and 310 to 360 below 369 classes, where they keep single FP32 loads.
 // For even n the diagonal is slower (176 to 209 ns; 277 when every row meets the odd one), so from
 // 369 classes on the array takes the graphs whose classes have at least 320 edges: at 232 the
@@ -1125,10 +1127,13 @@ cudaError_t lowd_sys_passes(lowd_ctx* h, int32_t passes) {
     const Geo g = make_geo(h->n);
     const bool weighted = h->w != nullptr;
     const bool pair = h->sys_pair != 0;
-    // one block when the pairs fit it (every stream then stays in shared memory).  Several: 1, 2,
-    // 3 and 4 pairs per block took 1,134, 1,025, 1,074 and 1,100 us on n = 9,109 and 302, 285, 301
-    // and 310 on 2,601 - fewer warps per SM are faster steps, more blocks are more slow hops.
-    const int W = g.KL <= (weighted ? kPairs : kMaxW) ? g.KL : kPairs;
+    // One block when the pairs fit it (every stream then stays in shared memory).  Of several, two
+    // pairs each for odd n while every SM holds one: fewer warps per SM are faster steps, more
+    // blocks are more slow hops.  Two against four pairs: n 513 59 against 64 us, 1,031 114 (124),
+    // 4,047 457 (489), weighted 460 (498), 9,109 1,066 (1,136); one pair 6 to 10 % slower than two.
+    // Even n gains nothing (770: 238 against 232 us, 9,110: 1,828 against 1,829) and keeps four.
+    const int several = (g.P == h->n && g.KL <= lowd_device_sms() * kPairsOdd) ? kPairsOdd : kPairs;
+    const int W = g.KL <= (weighted ? kPairs : kMaxW) ? g.KL : several;
     const int grid = (g.KL + W - 1) / W;
     size_t smem = (size_t)(2 * W + 1) * kRing * 16u + (size_t)W * (kOddBytes + 16u);
     if (grid == 1) smem += (size_t)(g.P + kPad) * 16u;
