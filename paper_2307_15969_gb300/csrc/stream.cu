@@ -130,47 +130,109 @@ __global__ void k_pending(const int32_t* __restrict__ pred, int64_t m, int32_t* 
 
 constexpr uint32_t kSpinLimit = 1u << 22;    // bounded waits: mbarrier try_wait rounds
 
+constexpr int kLevelT = 1024;         // threads of the level colouring, one block per SM
+constexpr int kLevelAlone = 4096;     // frontiers below this many ranks are left to one SM
+constexpr size_t kLevelSmem = 2 * (size_t)kLevelAlone * (sizeof(int2) + sizeof(int32_t));
+
 // Kahn's algorithm by levels.  ctl: [0..2] frontier sizes (rotating), [4] barrier count,
 // [5] barrier generation, [6] level count out.  Frontier r lives in fr[r & 1].  While the
-// frontier holds at least `small` ranks every block works on it and blocks meet at a grid
-// barrier per level; below that, block 0 goes on alone with block barriers.
-__global__ void k_levels(int32_t* __restrict__ pend, const int32_t* __restrict__ succ, int32_t* __restrict__ level,
-                         int32_t* __restrict__ f0, int32_t* __restrict__ f1, int32_t* __restrict__ ctl,
-                         int32_t small, int32_t* __restrict__ err) {
+// frontier holds at least kLevelAlone ranks every block works on it and blocks meet at a grid
+// barrier per level; from the first smaller one on, block 0 goes on alone with block barriers.
+//
+// The levels are a chain, one after the other, so what counts is one level's latency.  Alone, the
+// frontier and its size stay in shared memory with the successors of its ranks (what exceeds
+// kLevelAlone ranks goes to fr), and the successors of a rank are read while the decrement of its
+// pending count is on its way, so a level is one trip to L2 and a block barrier.
+// Measured (GB300; schedule 2's whole preparation, before with 256 threads, the frontier in global
+// memory and two blocks per SM): unpruned R-MAT scale 16, 9,727 levels, 25.9
+// -> 14.5 ms; scale 18, 25,313 levels, 55.9 -> 34.5; scale 20 weighted with hub stars, 4,833
+// levels, 38.5 -> 22.4.  1,024 threads a block alone gave 23.8, 47.8 and 25.4; leaving frontiers
+// below 2,048, 8,192 or 16,384 ranks to one SM made it 24.4, 28.0 and 29.6 on the last.
+__global__ void __launch_bounds__(kLevelT, 1)
+k_levels(int32_t* __restrict__ pend, const int2* __restrict__ succ, int32_t* __restrict__ level, int32_t* f0,
+         int32_t* f1, int32_t* ctl, int32_t* __restrict__ err) {
+    extern __shared__ int2 near_succ[];                       // [2][kLevelAlone]
+    int32_t* near_rank = (int32_t*)(near_succ + 2 * kLevelAlone);   // [2][kLevelAlone]
+    __shared__ int32_t size[3];
     int32_t* fr[2] = {f0, f1};
     volatile int32_t* vctl = ctl;
-    bool alone = false;
-    for (int32_t r = 0;; ++r) {
-        const int32_t ncur = vctl[r % 3];
-        if (ncur == 0) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) ctl[6] = r;
-            return;
-        }
-        if (!alone && ncur < small) {
-            if (blockIdx.x != 0) return;
-            alone = true;
-        }
+    int32_t r = 0, ncur;
+    for (;; ++r) {
+        ncur = vctl[r % 3];
+        if (ncur < kLevelAlone) break;
         const int32_t* cur = fr[r & 1];
         int32_t* nxt = fr[(r + 1) & 1];
         if (threadIdx.x == 0 && blockIdx.x == 0) ctl[(r + 2) % 3] = 0;   // the frontier after next
-        const int64_t stride = alone ? (int64_t)blockDim.x : (int64_t)gridDim.x * blockDim.x;
-        const int64_t t0 = alone ? (int64_t)threadIdx.x : (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-        for (int64_t i = t0; i < ncur; i += stride) {
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ncur;
+             i += (int64_t)gridDim.x * blockDim.x) {
             const int32_t k = cur[i];
             level[k] = r;
+            const int2 sc = succ[k];
 #pragma unroll
             for (int s = 0; s < 2; ++s) {
-                const int32_t t = succ[2 * (int64_t)k + s];
+                const int32_t t = s ? sc.y : sc.x;
                 if (t >= 0 && atomicSub(&pend[t], 1) == 1) nxt[atomicAdd(&ctl[(r + 1) % 3], 1)] = t;
             }
         }
-        if (alone) {
-            __threadfence_block();
-            __syncthreads();
-        } else if (!grid_barrier((unsigned*)&ctl[4], (volatile unsigned*)&ctl[5], gridDim.x, err)) {
-            return;
-        }
+        if (!grid_barrier((unsigned*)&ctl[4], (volatile unsigned*)&ctl[5], gridDim.x, err)) return;
     }
+    if (blockIdx.x != 0) return;
+    for (int32_t i = threadIdx.x; i < ncur; i += blockDim.x) {
+        const int32_t k = fr[r & 1][i];
+        near_rank[(r & 1) * kLevelAlone + i] = k;
+        near_succ[(r & 1) * kLevelAlone + i] = succ[k];
+    }
+    if (threadIdx.x < 3) size[threadIdx.x] = threadIdx.x == r % 3 ? ncur : 0;
+    __syncthreads();
+    while (ncur > 0) {
+        const int2* cur_succ = near_succ + (r & 1) * kLevelAlone;
+        const int32_t* cur_rank = near_rank + (r & 1) * kLevelAlone;
+        int2* nxt_succ = near_succ + ((r + 1) & 1) * kLevelAlone;
+        int32_t* nxt_rank = near_rank + ((r + 1) & 1) * kLevelAlone;
+        const int32_t* cur_far = fr[r & 1];
+        int32_t* nxt_far = fr[(r + 1) & 1];
+        int32_t* nxt_size = &size[(r + 1) % 3];
+        if (threadIdx.x == 0) size[(r + 2) % 3] = 0;
+        // whole warps at a time, so that a warp asks for its places in the next frontier once
+        for (int32_t base = (int32_t)threadIdx.x & ~31; base < ncur; base += blockDim.x) {
+            const int32_t i = base + (int32_t)lane_id();
+            int2 t = make_int2(-1, -1);
+            if (i < ncur) {
+                int32_t k;
+                if (i < kLevelAlone) {
+                    k = cur_rank[i];
+                    t = cur_succ[i];
+                } else {
+                    k = cur_far[i];
+                    t = succ[k];
+                }
+                level[k] = r;
+            }
+            int2 tx = t, ty = t;
+            int32_t px = 0, py = 0;
+            if (t.x >= 0) { px = atomicSub(&pend[t.x], 1); tx = succ[t.x]; }
+            if (t.y >= 0) { py = atomicSub(&pend[t.y], 1); ty = succ[t.y]; }
+            const unsigned bx = __ballot_sync(0xffffffffu, px == 1), by = __ballot_sync(0xffffffffu, py == 1);
+            if (!(bx | by)) continue;
+            int32_t at = 0;
+            if (lane_id() == 0) at = atomicAdd(nxt_size, __popc(bx) + __popc(by));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            const unsigned below = (1u << lane_id()) - 1u;
+            const int32_t ix = at + __popc(bx & below), iy = at + __popc(bx) + __popc(by & below);
+            if (px == 1) {
+                if (ix < kLevelAlone) { nxt_rank[ix] = t.x; nxt_succ[ix] = tx; }
+                else nxt_far[ix] = t.x;
+            }
+            if (py == 1) {
+                if (iy < kLevelAlone) { nxt_rank[iy] = t.y; nxt_succ[iy] = ty; }
+                else nxt_far[iy] = t.y;
+            }
+        }
+        __syncthreads();   // orders fr too: one block writes and reads it
+        ++r;
+        ncur = size[r % 3];
+    }
+    if (threadIdx.x == 0) ctl[6] = r;
 }
 
 // level of every rank; the class-major order is the ranks sorted by level, ascending in a level
@@ -957,15 +1019,13 @@ lowd_status lowd_stream_prepare(lowd_ctx* h, const float* init_splits_canon) {
             cudaMemsetAsync(ctl, 0, 16 * sizeof(int32_t), st);
             LOWD_LAUNCH(k_pending, grid_for(m), kT, 0, st, pred, m, pend, fr[0], ctl);
             // ---- 3. levels (cooperative: every block must be resident for the grid barrier)
-            int dev = 0, nb_per_sm = 0;
-            cudaGetDevice(&dev);
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb_per_sm, k_levels, kT, 0);
-            int nblocks = lowd_device_sms() * (nb_per_sm > 2 ? 2 : (nb_per_sm > 0 ? nb_per_sm : 1));
-            int32_t small = 4096;
             int32_t* errp = h->d_i32 + 10;
             cudaMemsetAsync(errp, 0, sizeof(int32_t), st);
-            void* args[] = {&pend, &succ, &level, &fr[0], &fr[1], &ctl, &small, &errp};
-            cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_levels, dim3(nblocks), dim3(kT), args, 0, st);
+            void* args[] = {&pend, &succ, &level, &fr[0], &fr[1], &ctl, &errp};
+            cudaError_t e = cudaFuncSetAttribute(k_levels, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLevelSmem);
+            if (e == cudaSuccess)
+                e = cudaLaunchCooperativeKernel((const void*)k_levels, dim3(lowd_device_sms()), dim3(kLevelT), args,
+                                                kLevelSmem, st);
             lowd_note_launch();
             if (e != cudaSuccess) { s = h->fail(e); break; }
             int32_t hc[8];
