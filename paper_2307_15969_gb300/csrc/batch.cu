@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(1024, 1) k_batch_lowd(BatchArgs A) {
     __shared__ int32_t s_graph, s_count, s_rem;
     __shared__ volatile int32_t s_bad;   // an edge id outside the core: recorded, never used
     __shared__ volatile int32_t s_abort; // a bounded wait of the staged passes expired
-    __shared__ int32_t s_stage_len;
+    __shared__ int32_t s_stage_len, s_longest;
     const int tid = threadIdx.x;
     const int nt = blockDim.x;
     for (;;) {
@@ -271,7 +271,13 @@ __global__ void __launch_bounds__(1024, 1) k_batch_lowd(BatchArgs A) {
         // ---------------- Algorithm 1 passes
         // Staged form: chunks of G consecutive classes move global -> shared through
         // cp.async.bulk (last warp), consumers update them in shared memory with a named
-        // barrier per class, splits go back by bulk stores.  Used when at least 3 stages of
+        // barrier per class, splits go back by bulk stores.  The classes are a chain, so a class's
+        // latency is what counts: only the warps that its longest class needs take part, and a
+        // thread reads its edge of the next class before the barrier, so that between two
+        // barriers lie the loads' read, the update and their write, without a branch.  256
+        // Chung-Lu graphs of up to 20,000 nodes, 100 passes: 22.5 -> 18.8 ms (21.8 with the fewer
+        // warps and the early read alone); the largest core (996 nodes, 250 edges a class) took
+        // 183 ns a class before.  Used when at least 3 stages of
         // the longest chunk fit and a pass has enough chunks for the store ordering;
         // otherwise classes are updated straight from global memory.
         const size_t used = (((4u * (size_t)(nH + 1) + 4u * (size_t)(P + 1)) + 7) & ~(size_t)7);
@@ -294,7 +300,10 @@ __global__ void __launch_bounds__(1024, 1) k_batch_lowd(BatchArgs A) {
                     break;
                 }
             }
-            if (tid == 0) { s_count = pick_g; s_rem = pick_s; s_stage_len = pick_len; }
+            int32_t longest = 0;
+            for (int32_t c = (int32_t)lane_id(); c < P; c += 32) longest = max(longest, start[c + 1] - start[c]);
+            longest = __reduce_max_sync(0xffffffffu, longest);
+            if (tid == 0) { s_count = pick_g; s_rem = pick_s; s_stage_len = pick_len; s_longest = longest; }
         }
         fence_proxy_async_all();   // the class-major edges and splits are read by bulk copies
         __syncthreads();
@@ -304,7 +313,9 @@ __global__ void __launch_bounds__(1024, 1) k_batch_lowd(BatchArgs A) {
             uint64_t* full = reinterpret_cast<uint64_t*>(sm + used);
             uint64_t* empty = full + S;
             unsigned char* stages = sm + stage_base;
-            const int nc = nt - 32;
+            const int nc = nt - 32;                                          // the producer's first thread
+            const int na = min(nc, max(32, (s_longest + 31) & ~31));         // consumers
+            const bool wide = s_longest > na;                                // more edges than consumers
             if (tid == 0) {
                 s_abort = 0;
                 for (int k = 0; k < S; ++k) { mbar_init(&full[k], 1); mbar_init(&empty[k], 1); }
@@ -354,7 +365,7 @@ __global__ void __launch_bounds__(1024, 1) k_batch_lowd(BatchArgs A) {
                     if (q < PT) drain_fills(full, S, q, pf, kBWaitLimit);
                     bulk_wait<0>();
                 }
-            } else {
+            } else if (tid < na) {
                 auto wait_full = [&](int32_t kk, uint32_t par) -> bool {
                     uint32_t spins = 0;
                     bool ok = mbar_try_wait(&full[kk], par);
@@ -363,7 +374,7 @@ __global__ void __launch_bounds__(1024, 1) k_batch_lowd(BatchArgs A) {
                 };
                 bool bad = false;
                 if (tid < 32 && PT > 0) bad = !wait_full(0, 0);
-                bad = consumer_sync_or(nc, bad);
+                bad = consumer_sync_or(na, bad);
                 int32_t k = 0, j = 0;
                 uint32_t parity = 0;
                 for (int32_t q = 0; q < PT && !bad; ++q) {
@@ -373,25 +384,53 @@ __global__ void __launch_bounds__(1024, 1) k_batch_lowd(BatchArgs A) {
                     unsigned char* st = stages + 2 * arr * (size_t)k;
                     const uint32_t* suv = reinterpret_cast<const uint32_t*>(st);
                     float* ss = reinterpret_cast<float*>(st + arr);
-                    int32_t cb = 0;
+                    auto update = [&](uint32_t p, float sv, int32_t r) {
+                        const int32_t a = (int32_t)(p & 0xffffu), b = (int32_t)(p >> 16);
+                        if (a > nH || b > nH) { s_bad = 1; return; }   // never taken: ids checked
+                        const float la = L[a], lb = L[b];
+                        const float diff = la - lb;
+                        const bool gt = diff > 0.0f;
+                        const float cap = gt ? sv : (1.0f - sv);
+                        const float d = fminf(fabsf(diff) * 0.5f, cap);
+                        const float dd = gt ? d : -d;
+                        L[a] = la - dd;
+                        L[b] = lb + dd;
+                        ss[r] = fminf(sv - dd, 1.0f);
+                    };
+                    // this thread's edge of a class: its ends and split, or the padding's node (a
+                    // no-op) where it has none
+                    auto fetch = [&](int32_t r, int32_t end, int32_t& a, int32_t& b, float& sv) {
+                        uint32_t p = sentinel;
+                        sv = 0.0f;
+                        if (r < end) { p = suv[r]; sv = ss[r]; }
+                        a = (int32_t)(p & 0xffffu);
+                        b = (int32_t)(p >> 16);
+                    };
+                    // class c is [cb, ce), the next one [ce, e1)
+                    int32_t cb = 0, ce = start[c0 + 1] - base, e1 = start[min(c0 + 2, c1)] - base;
+                    int32_t a, b;
+                    float sv;
+                    fetch(tid, ce, a, b, sv);
                     for (int32_t c = c0; c < c1; ++c) {
-                        const int32_t ce = start[c + 1] - base;
-                        for (int32_t r = cb + tid; r < ce; r += nc) {
-                            const uint32_t p = suv[r];
-                            const int32_t a = (int32_t)(p & 0xffffu), b = (int32_t)(p >> 16);
-                            if (a > nH || b > nH) { s_bad = 1; continue; }   // never taken: ids checked
-                            const float la = L[a], lb = L[b], sv = ss[r];
-                            const float diff = la - lb;
-                            const bool gt = diff > 0.0f;
-                            const float cap = gt ? sv : (1.0f - sv);
-                            const float d = fminf(fabsf(diff) * 0.5f, cap);
-                            const float dd = gt ? d : -d;
-                            L[a] = la - dd;
-                            L[b] = lb + dd;
-                            ss[r] = fminf(sv - dd, 1.0f);
-                        }
-                        cb = ce;
-                        if (c + 1 < c1) consumer_sync(nc);
+                        if (a > nH || b > nH) { s_bad = 1; a = b = nH; }   // never taken: ids checked
+                        const float la = L[a], lb = L[b];
+                        const int32_t e2 = start[min(c + 3, c1)] - base;
+                        int32_t an, bn;
+                        float svn;
+                        fetch(ce + tid, e1, an, bn, svn);
+                        const float diff = la - lb;
+                        const bool gt = diff > 0.0f;
+                        const float cap = gt ? sv : (1.0f - sv);
+                        const float d = fminf(fabsf(diff) * 0.5f, cap);
+                        const float dd = gt ? d : -d;
+                        L[a] = la - dd;
+                        L[b] = lb + dd;
+                        if (cb + tid < ce) ss[cb + tid] = fminf(sv - dd, 1.0f);
+                        if (wide)
+                            for (int32_t r = cb + tid + na; r < ce; r += na) update(suv[r], ss[r], r);
+                        cb = ce; ce = e1; e1 = e2;
+                        a = an; b = bn; sv = svn;
+                        if (c + 1 < c1) consumer_sync(na);
                     }
                     fence_proxy_async_smem();
                     const int32_t kprev = k;
@@ -399,7 +438,7 @@ __global__ void __launch_bounds__(1024, 1) k_batch_lowd(BatchArgs A) {
                     j = (j + 1 == NC) ? 0 : j + 1;
                     bool fail = false;
                     if (tid < 32 && q + 1 < PT) fail = !wait_full(k, parity);
-                    bad = consumer_sync_or(nc, fail);
+                    bad = consumer_sync_or(na, fail);
                     if (tid == 0) mbar_arrive(&empty[kprev]);
                 }
                 if (bad && tid == 0) s_abort = 1;
