@@ -53,13 +53,30 @@ def _peaks():
     return 6800.0, "fallback"
 
 
-def _sweep_hash():
-    """Hash of the staged sweep kernel's source: its layout, the kernel and its launcher."""
-    with open(os.path.join(ROOT, "paper_2307_15969_gb300", "csrc", "sweep.cu")) as f:
+# per pass kernel of schedule 1: its source file, the spans hashed (kernel and launcher, to its
+# closing brace) and its committed ncu record
+RECORDS = {
+    "k_sweep_tma": ("sweep.cu", (("struct TmaLayout {", "// The same staging as k_sweep_tma"),
+                                 ("cudaError_t launch_sweep_tma(", "\n}\n")), "k_sweep_tma_rmat22_dram.json"),
+    "k_sweep_systolic": ("systolic.cu", (("k_sweep_systolic(const SysArgs a) {", "\n}\n"),
+                                         ("cudaError_t lowd_sys_passes(", "\n}\n")),
+                         "k_sweep_systolic_rmat22_dram.json"),
+}
+
+
+def _pass_kernel(n, m, classes):
+    """The kernel that runs a schedule-1 pass over a core of pair loads: the array serves odd n,
+    and even n from 320 edges a class on (the rule of lowd_sys_serves, for cores whose cells are
+    within 16 per edge)."""
+    return "k_sweep_systolic" if n % 2 or m >= 320 * classes else "k_sweep_tma"
+
+
+def _sweep_hash(kernel="k_sweep_tma"):
+    """Hash of a pass kernel's source: the kernel and its launcher."""
+    with open(os.path.join(ROOT, "paper_2307_15969_gb300", "csrc", RECORDS[kernel][0])) as f:
         s = f.read()
     parts = []
-    for a, b in (("struct TmaLayout {", "// The same staging as k_sweep_tma"),
-                 ("cudaError_t launch_sweep_tma(", "\n}\n")):   # the launcher, to its closing brace
+    for a, b in RECORDS[kernel][1]:
         i = s.find(a)
         j = s.find(b, i) if i >= 0 else -1
         if i < 0 or j < i:
@@ -68,21 +85,21 @@ def _sweep_hash():
     return hashlib.sha256("".join(parts).encode()).hexdigest()[:16]
 
 
-def _sweep_record():
-    """The committed ncu record of the staged sweep (DRAM bytes per pass, warp instructions
-    per class), if it was taken on the current sweep kernel source."""
-    p = os.path.join(ROOT, "profiles", "k_sweep_tma_rmat22_dram.json")
+def _sweep_record(kernel="k_sweep_tma"):
+    """The committed ncu record of a pass kernel (DRAM bytes per pass, warp instructions per
+    class), if it was taken on the current source of the kernel."""
+    p = os.path.join(ROOT, "profiles", RECORDS[kernel][2])
     if not os.path.exists(p):
         return None
     with open(p) as f:
         d = json.load(f)
-    if d.get("sweep_cu_sha256_16") != _sweep_hash():
+    if d.get("sweep_cu_sha256_16") != _sweep_hash(kernel):
         return None
     return d
 
 
-def _traffic_per_pass():
-    d = _sweep_record()
+def _traffic_per_pass(kernel="k_sweep_tma"):
+    d = _sweep_record(kernel)
     return float(d["dram_bytes_per_pass"]) if d else None
 
 
@@ -669,12 +686,12 @@ def main():
         return 0
 
     achieved = BYTES_PER_UPDATE * m_H * T / sweep_s / 1e9
-    tpp = _traffic_per_pass()
-    rec = _sweep_record()
-    mhz = ck.get("sm_mhz") if isinstance(ck, dict) else None
-    issue_floor = (rec["warp_instructions_per_class"] / 4.0 / (mhz * 1e6) * 1e9
-                   if rec and rec.get("warp_instructions_per_class") and mhz else None)
     C = info["classes"]
+    kernel = _pass_kernel(info["n_H"], m_H, C)
+    tpp = _traffic_per_pass(kernel)
+    rec = _sweep_record(kernel)
+    if rec and args.workload not in rec["workload"]:
+        rec = tpp = None             # DRAM bytes of another graph
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": total / args.steps * 1e3, "higher_is_better": True,
@@ -686,16 +703,14 @@ def main():
                    "l2": "flushed between timed steps (256 MB write); G's edge arrays (537 MB) exceed L2"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": (tpp * T if tpp is not None else None),
-                     "kernel": "k_sweep_tma", "peak_kind": peak_kind,
+                     "kernel": kernel, "peak_kind": peak_kind,
                      "launch_ms": sweep_s * 1e3, "bytes_per_update": BYTES_PER_UPDATE,
                      "sweep_kernel": info["sweep_kernel"], "edges_per_thread": info["edges_per_thread"],
                      "chain": {"classes_per_pass": C, "ns_per_class": sweep_s / T / max(C, 1) * 1e9,
-                               "issue_floor_ns_per_class": issue_floor,
-                               "note": "each class waits for the previous one (Delta(H) >= n_H - 3 "
-                                       "classes on this near-clique core): the pass is bound by the "
-                                       "per-class chain on one SM, not by HBM; the issue floor is "
-                                       "the class's warp instructions (ncu) over 4 schedulers at "
-                                       "the sampled SM clock"}},
+                               "note": "each class waits for the previous one at their common "
+                                       "nodes (Delta(H) >= n_H - 3 classes on this near-clique "
+                                       "core): the pass is bound by the chain of classes, not by "
+                                       "HBM"}},
         "e2e": {"value": m_H * T / e2e_s, "unit": UNIT, "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h, "ms_per_step": e2e_s * 1e3},
         "stages_ms": stages,

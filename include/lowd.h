@@ -71,16 +71,16 @@ typedef struct {
     double  rel_tol;      /* >0: stop once (D - rho(S))/rho(S) <= rel_tol at a check, where
                              D = max load (an upper bound on rho*, Sec. III-B) and S the
                              best prefix of the load order (default 0: run all k passes) */
-    int32_t schedule;     /* 0 = automatic; 1 = one-CTA shared-memory sweep (node count
-                             must fit shared memory); 2 = grid sweep over matchings */
+    int32_t schedule;     /* 0 = automatic; 1 = circle colouring (node count must fit one SM's
+                             shared memory); 2 = level order (any size) */
     int32_t rederive_every; /* re-derive the FP32 loads from the splits (FP64 sums) after at
                              most this many passes, bounding the drift of the running FP32
                              loads: 0 = default 50, < 0 = only at the end of the call */
     int32_t node_versions; /* 1: the one-CTA staged sweep replaces its barrier after every
                              colour class by per-node versions (kernel 5: an update waits only
                              for the previous updates of its two nodes); same pass as kernel 1.
-                             Default 0 (kernel 1: on dense cores whose hubs appear in every
-                             class it is faster, as waiting warps sleep at the barrier) */
+                             Default 0: the passes run as wavefronts over many SMs where that
+                             is faster, else in the one-CTA staged sweep */
     int32_t hub_stars;    /* hub-star block updates (read when the schedule is built, i.e. by
                              the first lowd_iterate of a graph; a schedule built earlier by
                              lowd_set_splits or lowd_warm_start has none): 0 = off (default); 1 =
@@ -128,15 +128,17 @@ typedef struct {
     int32_t weighted;     /* 1 if weights were given */
     int32_t pruned;       /* 1 after lowd_prune */
     int32_t classes;      /* colour classes of the schedule (0 before lowd_iterate) */
-    int32_t schedule;     /* schedule in use: 1 one-CTA shared memory, 2 grid matchings */
+    int32_t schedule;     /* schedule in use: 1 circle colouring, 2 level order */
     int32_t max_degree;   /* maximum (unweighted) degree of the current graph */
     int32_t prune_rounds; /* rounds lowd_prune ran */
-    int32_t sweep_kernel; /* kernel of the last pass: 0 none yet, 1 staged one-CTA sweep with
-                             pair loads and a barrier per class, 2 one-CTA register-ring sweep,
-                             3 one-CTA simple sweep, 4 streamed sweep (schedule 2, loads in
-                             global memory), 5 staged one-CTA sweep with pair loads and
+    int32_t sweep_kernel; /* kernel of the last pass, by its arithmetic: 0 none yet, 1 pair loads
+                             (wavefronts over the GPU, or the staged one-CTA sweep with a barrier
+                             per class), 2 single FP32 loads (wavefronts, or the one-CTA
+                             register-ring sweep), 3 one-CTA simple sweep, 4 streamed sweep
+                             (schedule 2, loads in global memory), 5 staged one-CTA sweep with pair loads and
                              per-node versions instead of class barriers */
-    int32_t sweep_edges_per_thread; /* edges per consumer thread per class of kernel 1 */
+    int32_t sweep_edges_per_thread; /* edges per consumer thread per class of the staged
+                                       sweep of this schedule (kernel 1) */
     int32_t star_threshold; /* hub degree threshold of the hub stars in use (0: none) */
     int32_t star_steps;     /* star steps per pass (the last star_steps entries of classes) */
     int32_t stars;          /* stars over all steps */
@@ -457,8 +459,8 @@ const char* lowd_last_error(lowd_handle h);
  * all threads).  A diagnostic for benchmarks; it has no counterpart in the paper. */
 uint64_t lowd_launch_count(void);
 
-/* Failure-detection self-test of the bounded grid barrier that the cooperative kernels (grid
- * steps of the streamed schedule, star steps, level colouring) meet at between steps: two
+/* Failure-detection self-test of the bounded grid barrier that the cooperative kernels (prune
+ * rounds, star steps, level colouring) meet at between steps: two
  * blocks are launched on a barrier that expects three, so nothing opens it; with a short spin
  * limit the wait must expire, set bit 1 (value 2) of the kernel's error word and end the
  * kernel.  *err_bits receives that word; returns LOWD_OK once the kernel has ended (the

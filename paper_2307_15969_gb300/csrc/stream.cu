@@ -11,9 +11,9 @@
 // max d classes (exactly max d on the R-MAT graphs, whose tail is the top hub's star).  The
 // levels are computed on the GPU by Kahn's algorithm, one frontier per level.
 //
-// Execution.  One CTA runs the classes in order; the loads of all n nodes stay in global
-// memory (L2) as FP32 pairs (hi, lo) moved by error-free transfers, as in the shared-memory
-// sweep.  The class-major edge stream is cut into chunks (at most kSegs classes or class
+// Execution.  The loads of all n nodes stay in global memory (L2) as FP32 pairs (hi, lo) moved by
+// error-free transfers.  The leading classes, which hold most edges, run over all SMs, ordered by
+// the tags of the node entries (k_sweep_nodes); one CTA runs the rest, in order.  Its class-major edge stream is cut into chunks (at most kSegs classes or class
 // pieces and at most Emax edges); producer warps stage each chunk in a ring of S shared-
 // memory stages: the ends, splits, weights and two 32-bit read descriptors by bulk copies,
 // and the two end loads of every edge by 8-byte cp.async gathers, D chunks ahead.  A load

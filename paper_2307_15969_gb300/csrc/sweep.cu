@@ -14,7 +14,8 @@
 // path serves are dense cores (maximum degree close to n), where P is within a few
 // colours of the lower bound Delta.
 //
-// Execution.  One CTA keeps every node load in shared memory for all passes of a call, as
+// Execution.  Where it is the faster one, the passes run as wavefronts over many SMs
+// (systolic.cu).  Otherwise one CTA keeps every node load in shared memory for all passes of a call, as
 // an FP32 pair (hi, lo) updated by error-free transfers (TwoSum), so no update rounds a load.
 // The class segments (packed 16-bit endpoint pairs when n <= 65536, the FP32 split and, if
 // weighted, the FP32 weight) are staged global -> shared in chunks of consecutive classes by
