@@ -549,25 +549,44 @@ k_sweep_tma(int32_t n, int32_t C, const int32_t* __restrict__ coff, const uint32
         float* ss = reinterpret_cast<float*>(st + lay.arr_bytes);
         const float* sw = reinterpret_cast<const float*>(st + 2 * lay.arr_bytes);
         int32_t cb = 0;
-        for (int32_t c = c0; c < c1; ++c) {
-            const int32_t ce = __shfl_sync(0xffffffffu, off_cur, c - c0 + 1) - base;
-            if (E == 1) {
-                // one edge per thread: the class fits the consumer threads
-                const int32_t r = cb + tid;
-                if (r < ce) {
-                    const uint32_t uv = suv[r];
-                    float2* pa = L + end_a(uv);
-                    float2* pb = L + end_b(uv);
-                    float2 A = *pa, Bv = *pb;
-                    const float ns = comp_transfer(A, Bv, ss[r], WEIGHTED ? sw[r] : 1.0f);
-                    *pa = A;
-                    *pb = Bv;
-                    ss[r] = ns;
+        if (E == 1) {
+            // One edge per thread (the class fits the consumer threads): its ends, split and
+            // weight are read before the barrier of its class, and a thread without an edge
+            // updates the padding's node, so that between two barriers lie the loads' read, the
+            // update and their write, without a branch (n 4,048, 254 edges a class: 174 -> 159 ns a
+            // class; n 6,194 weighted 192 -> 165).
+            auto fetch = [&](int32_t r, int32_t end, uint32_t& uv, float& sv, float& wv) {
+                uv = (uint32_t)n | ((uint32_t)n << 16);
+                sv = 0.0f;
+                wv = WEIGHTED ? 0.0f : 1.0f;
+                if (r < end) {
+                    uv = suv[r];
+                    sv = ss[r];
+                    if (WEIGHTED) wv = sw[r];
                 }
-                cb = ce;
+            };
+            int32_t ce = __shfl_sync(0xffffffffu, off_cur, 1) - base;
+            uint32_t uv;
+            float sv, wv;
+            fetch(tid, ce, uv, sv, wv);
+            for (int32_t c = c0; c < c1; ++c) {
+                float2* pa = L + end_a(uv);
+                float2* pb = L + end_b(uv);
+                float2 A = *pa, Bv = *pb;
+                const int32_t e1 = __shfl_sync(0xffffffffu, off_cur, min(c + 2, c1) - c0) - base;
+                uint32_t uvn;
+                float svn, wvn;
+                fetch(ce + tid, e1, uvn, svn, wvn);
+                const float ns = comp_transfer(A, Bv, sv, wv);
+                *pa = A;
+                *pb = Bv;
+                if (cb + tid < ce) ss[cb + tid] = ns;
+                cb = ce; ce = e1;
+                uv = uvn; sv = svn; wv = wvn;
                 if (c + 1 < c1) consumer_sync(nc);
-                continue;
             }
+        } else for (int32_t c = c0; c < c1; ++c) {
+            const int32_t ce = __shfl_sync(0xffffffffu, off_cur, c - c0 + 1) - base;
             for (int32_t r0 = cb + tid; r0 < ce; r0 += E * nc) {
                 uint32_t uv[E];
                 EdgeVal e[E];

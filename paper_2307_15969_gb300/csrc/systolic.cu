@@ -1040,7 +1040,8 @@ lowd_status lowd_sys_class_sizes(lowd_ctx* h, const int32_t* u, const int32_t* v
 // 297 (710) and 933 (2,090), and 310 to 360 below 369 classes, where they keep single FP32 loads.
 // For even n the diagonal is slower (176 to 209 ns; 277 when every row meets the odd one), so from
 // 369 classes on the array takes the graphs whose classes have at least 320 edges: at 232 the
-// staged sweep is still ahead (175 against 203 ns), at 402 it is not (215 against 195).
+// staged sweep is still ahead (175 against 203 ns), at 402 it is not (215 against 195; its edges
+// have been read a class early since: 174 -> 159 ns at n 4,048).
 bool lowd_sys_serves(int32_t n, int64_t m, int32_t C, bool pair) {
     if (n < 9) return false;
     const Geo g = make_geo(n);
