@@ -436,7 +436,7 @@ __device__ __forceinline__ void store_split(const Tile& t, int32_t s, uint32_t s
     }
 }
 
-// until the entry of step s is in the ring: polls it alone (the entries come in order)
+// until the entry of step s is in the ring: polls it alone
 template <bool PAIR>
 __device__ __forceinline__ void poll_entry(const Tile& t, int32_t s, const Bad& w, bool& bad) {
     const uint32_t at = t.ring + ((((uint32_t)s + t.in_off) & t.rmask) << 4);
@@ -448,18 +448,19 @@ __device__ __forceinline__ void poll_entry(const Tile& t, int32_t s, const Bad& 
     }
 }
 
-// until the entries j0 .. j1 - 1 of the group at step s0 (EDGE: those that exist) are in t.e
+// until the entries j0 .. j1 - 1 of the group at step s0 (EDGE: those that exist) are in t.e.  The tag
+// of every one of them is looked at: they mostly come in order, so it is the last one that is
+// polled, but the wrap's come from the warps of different tiles, and nothing orders those.
 template <bool PAIR, bool EDGE>
 __device__ __forceinline__ void await_entries(Tile& t, int32_t s0, int j0, int j1, const Bad& w, bool& bad) {
-    if (EDGE && s0 + j1 > t.in_end) {      // the inputs run out inside the group
-        if (s0 + j0 >= t.in_end) return;
-        poll_entry<PAIR>(t, t.in_end - 1, w, bad);
-        read_ahead<PAIR>(t, s0);
-        return;
+    if (EDGE) {                            // the inputs may run out inside the group
+        j1 = min(j1, t.in_end - s0);
+        if (j1 <= j0) return;
     }
-    while (__any_sync(0xffffffffu, missing<PAIR>(t, s0, j0, j1) != 0u) && !bad) {
+    for (uint32_t spins = 1; __any_sync(0xffffffffu, missing<PAIR>(t, s0, j0, j1) != 0u) && !bad; ++spins) {
         poll_entry<PAIR>(t, s0 + j1 - 1, w, bad);
         read_ahead<PAIR>(t, s0);
+        if ((spins & 255u) == 255u) bad = __any_sync(0xffffffffu, bad || w.expired(spins, kSpinSmem));
     }
 }
 
