@@ -415,6 +415,9 @@ constexpr int kStoreSlack = 1;    // bulk stores allowed to be still reading the
 constexpr int kStoreGroups = 8;   // bulk stores allowed in flight at all
 constexpr uint32_t kWaitLimit = 1u << 22;   // try_wait rounds before giving up
 constexpr int32_t kTmaMinClasses = 369;     // fewest classes it runs on (16 per chunk, 16 stages)
+// Dynamic shared memory of a staged sweep at most: a block's 227 KB less its static word, which takes
+// 128 bytes before the 128-byte aligned dynamic part.
+constexpr size_t kStagedSmemMost = 227 * 1024 - 128;
 
 struct TmaLayout {
     uint32_t bars, L, CO, stages, stage_bytes, arr_bytes, total;
@@ -910,7 +913,7 @@ struct TmaPick {
 };
 
 TmaPick tma_pick(const lowd_ctx* h, bool weighted) {
-    constexpr size_t budget = 227 * 1024;
+    constexpr size_t budget = kStagedSmemMost;
     constexpr int kMinStages = 3;
     TmaPick p;
     for (int32_t g : {16, 8, 4, 2, 1}) {
@@ -1008,7 +1011,7 @@ struct FlowPick {
 };
 
 FlowPick flow_pick(const lowd_ctx* h, bool weighted, int32_t maxlen) {
-    constexpr size_t budget = 227 * 1024;
+    constexpr size_t budget = kStagedSmemMost;
     constexpr int kMinStages = 3;
     FlowPick p;
     if (maxlen > kTmaConsumers) return p;
