@@ -64,11 +64,12 @@ RECORDS = {
 }
 
 
-def _pass_kernel(n, m, classes):
-    """The kernel that runs a schedule-1 pass over a core of pair loads: the array serves odd n,
-    and even n from 320 edges a class on (the rule of lowd_sys_serves, for cores whose cells are
-    within 16 per edge)."""
-    return "k_sweep_systolic" if n % 2 or m >= 320 * classes else "k_sweep_tma"
+def _pass_kernel(info):
+    """The kernel that ran the last pass, by lowd_info."""
+    if info["wavefront_blocks"]:
+        return "k_sweep_systolic"
+    return {1: "k_sweep_tma", 2: "k_sweep_vec", 3: "k_sweep_simple", 4: "k_sweep_stream",
+            5: "k_sweep_flow"}.get(info["sweep_kernel"])
 
 
 def _sweep_hash(kernel="k_sweep_tma"):
@@ -88,6 +89,8 @@ def _sweep_hash(kernel="k_sweep_tma"):
 def _sweep_record(kernel="k_sweep_tma"):
     """The committed ncu record of a pass kernel (DRAM bytes per pass, warp instructions per
     class), if it was taken on the current source of the kernel."""
+    if kernel not in RECORDS:
+        return None
     p = os.path.join(ROOT, "profiles", RECORDS[kernel][2])
     if not os.path.exists(p):
         return None
@@ -528,7 +531,8 @@ def main():
         info_ = pkg.lowd_get_info(h)
         stats.update(n_H=nk, m_H=mk, rounds=rounds, rho=rho, S=int(S.shape[0]),
                      classes=info_["classes"], sweep_kernel=info_["sweep_kernel"],
-                     edges_per_thread=info_["sweep_edges_per_thread"])
+                     edges_per_thread=info_["sweep_edges_per_thread"],
+                     wavefront_blocks=info_["wavefront_blocks"])
         pkg.lowd_free(h)
 
     peak, peak_kind = _peaks()
@@ -687,7 +691,7 @@ def main():
 
     achieved = BYTES_PER_UPDATE * m_H * T / sweep_s / 1e9
     C = info["classes"]
-    kernel = _pass_kernel(info["n_H"], m_H, C)
+    kernel = _pass_kernel(info)
     tpp = _traffic_per_pass(kernel)
     rec = _sweep_record(kernel)
     if rec and args.workload not in rec["workload"]:
@@ -706,6 +710,7 @@ def main():
                      "kernel": kernel, "peak_kind": peak_kind,
                      "launch_ms": sweep_s * 1e3, "bytes_per_update": BYTES_PER_UPDATE,
                      "sweep_kernel": info["sweep_kernel"], "edges_per_thread": info["edges_per_thread"],
+                     "wavefront_blocks": info["wavefront_blocks"],
                      "chain": {"classes_per_pass": C, "ns_per_class": sweep_s / T / max(C, 1) * 1e9,
                                "note": "each class waits for the previous one at their common "
                                        "nodes (Delta(H) >= n_H - 3 classes on this near-clique "

@@ -134,14 +134,17 @@ typedef struct {
     int32_t sweep_kernel; /* kernel of the last pass, by its arithmetic: 0 none yet, 1 pair loads
                              (wavefronts over the GPU, or the staged one-CTA sweep with a barrier
                              per class), 2 single FP32 loads (wavefronts, or the one-CTA
-                             register-ring sweep), 3 one-CTA simple sweep, 4 streamed sweep
+                             register-ring sweep; wavefront_blocks tells them apart), 3 one-CTA simple sweep, 4 streamed sweep
                              (schedule 2, loads in global memory), 5 staged one-CTA sweep with pair loads and
                              per-node versions instead of class barriers */
     int32_t sweep_edges_per_thread; /* edges per consumer thread per class of the staged
-                                       sweep of this schedule (kernel 1) */
+                                       sweep (kernel 1; where wavefronts ran instead, of the
+                                       staged sweep that these classes would take) */
     int32_t star_threshold; /* hub degree threshold of the hub stars in use (0: none) */
     int32_t star_steps;     /* star steps per pass (the last star_steps entries of classes) */
     int32_t stars;          /* stars over all steps */
+    int32_t wavefront_blocks; /* thread blocks of the wavefronts that ran the last pass's plain
+                                 edges; 0: another kernel ran them, or no pass yet */
     int64_t star_edges;     /* star edges (the rest, m - star_edges, run Algorithm 1) */
 } lowd_info;
 

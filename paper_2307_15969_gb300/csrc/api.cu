@@ -361,6 +361,7 @@ lowd_status lowd_get_info(lowd_handle h, lowd_info* info) {
     x.star_threshold = h->star_tau;
     x.star_steps = h->star_S;
     x.stars = h->star_nseg;
+    x.wavefront_blocks = h->wave_blocks;
     x.star_edges = h->star_m;
     *info = x;
     return LOWD_OK;

@@ -1114,6 +1114,7 @@ cudaError_t run_plain(lowd_ctx* h, int32_t passes) {
         h->sweep_E = h->sys_pair ? tma_edges_per_thread(longest_class(h)) : 0;
         return lowd_sys_passes(h, passes);
     }
+    h->wave_blocks = 0;
     return h->cw ? launch_sweep<true>(h, passes) : launch_sweep<false>(h, passes);
 }
 

@@ -1137,6 +1137,7 @@ cudaError_t lowd_sys_passes(lowd_ctx* h, int32_t passes) {
     const int several = (g.P == h->n && g.KL <= lowd_device_sms() * kPairsOdd) ? kPairsOdd : kPairs;
     const int W = g.KL <= (weighted ? kPairs : kMaxW) ? g.KL : several;
     const int grid = (g.KL + W - 1) / W;
+    h->wave_blocks = grid;
     size_t smem = (size_t)(2 * W + 1) * kRing * 16u + (size_t)W * (kOddBytes + 16u);
     if (grid == 1) smem += (size_t)(g.P + kPad) * 16u;
     const size_t arrays = weighted ? 2u : 1u;

@@ -68,7 +68,8 @@ class lowd_info(C.Structure):
                 ("classes", C.c_int32), ("schedule", C.c_int32), ("max_degree", C.c_int32),
                 ("prune_rounds", C.c_int32), ("sweep_kernel", C.c_int32),
                 ("sweep_edges_per_thread", C.c_int32), ("star_threshold", C.c_int32),
-                ("star_steps", C.c_int32), ("stars", C.c_int32), ("star_edges", C.c_int64)]
+                ("star_steps", C.c_int32), ("stars", C.c_int32), ("wavefront_blocks", C.c_int32),
+                ("star_edges", C.c_int64)]
 
 
 class lowd_batch_options(C.Structure):
