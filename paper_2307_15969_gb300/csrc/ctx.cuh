@@ -191,7 +191,8 @@ lowd_status lowd_sweep_load_canonical(lowd_ctx* h, const float* splits_dev);
 lowd_status lowd_sweep_edge_order(lowd_ctx* h, int32_t* out_dev);
 
 // systolic.cu
-bool lowd_sys_serves(int32_t n, int64_t m, int32_t C, bool pair);
+bool lowd_sys_may_serve(int32_t n, int64_t m);
+bool lowd_sys_serves(int32_t n, int64_t m, int32_t C, int32_t longest, int64_t odd_edges, bool pair);
 lowd_status lowd_sys_class_sizes(lowd_ctx* h, const int32_t* u, const int32_t* v, int64_t m, int32_t* cnt_h);
 lowd_status lowd_sys_build(lowd_ctx* h, const int32_t* plain_ids, int64_t m_plain, const float* init_splits_canon);
 lowd_status lowd_sys_rederive(lowd_ctx* h, double* L64);

@@ -414,7 +414,6 @@ constexpr int kTmaMaxStages = 16;
 constexpr int kStoreSlack = 1;    // bulk stores allowed to be still reading their stage
 constexpr int kStoreGroups = 8;   // bulk stores allowed in flight at all
 constexpr uint32_t kWaitLimit = 1u << 22;   // try_wait rounds before giving up
-constexpr int32_t kTmaMinClasses = 369;     // fewest classes it runs on (16 per chunk, 16 stages)
 // Dynamic shared memory of a staged sweep at most: a block's 227 KB less its static word, which takes
 // 128 bytes before the 128-byte aligned dynamic part.
 constexpr size_t kStagedSmemMost = 227 * 1024 - 128;
@@ -1145,9 +1144,8 @@ static lowd_status prepare_systolic(lowd_ctx* h, const StarSplit& sp, const floa
     const int64_t mc = sp.pid ? sp.m_plain : h->m;
     if (mc == 0 || h->use_versions) return LOWD_OK;
     const int32_t P = h->n + (h->n & 1) - 1;
-    // no need to count the classes of a graph that would not be served with half of them
-    if (!lowd_sys_serves(h->n, mc, P / 2, P > 2 * kTmaMinClasses)) return LOWD_OK;
-    std::vector<int32_t> cnt((size_t)P), real;
+    if (!lowd_sys_may_serve(h->n, mc)) return LOWD_OK;
+    std::vector<int32_t> cnt((size_t)P + 1), real;
     LOWD_TRY(lowd_sys_class_sizes(h, sp.pid ? sp.gu : h->u, sp.pid ? sp.gv : h->v, mc, cnt.data()));
     real.reserve((size_t)P + 1);
     real.push_back(0);
@@ -1162,7 +1160,7 @@ static lowd_status prepare_systolic(lowd_ctx* h, const StarSplit& sp, const floa
         h->coff_h[c + 1] = h->coff_h[c] + ((real[(size_t)c + 1] - real[(size_t)c] + 3) & ~3);
     h->C = C;
     h->sys_pair = tma_pick(h, h->w != nullptr).G > 0 ? 1 : 0;
-    const bool serves = lowd_sys_serves(h->n, mc, C, h->sys_pair != 0);
+    const bool serves = lowd_sys_serves(h->n, mc, C, longest_class(h), cnt[(size_t)P], h->sys_pair != 0);
     const lowd_status b = serves ? lowd_sys_build(h, sp.pid, mc, init_splits_canon) : LOWD_ERR_OUT_OF_MEMORY;
     if (b != LOWD_OK) {   // not served, or no memory for the cells: the class-major kernels need less
         dfree(h, &h->sys_cs); dfree(h, &h->sys_cw); dfree(h, &h->sys_ids);

@@ -1003,10 +1003,13 @@ __device__ __forceinline__ int32_t circle_colour(int32_t P, int32_t a, int32_t b
     return a >= P ? a - P : a;   // a + b < 2P and 2a < 2P
 }
 
+// class sizes into cnt [0, P), the edges at the odd one into cnt [P]
 __global__ void k_colour_counts(int32_t P, const int32_t* __restrict__ u, const int32_t* __restrict__ v, int64_t m,
                                 int32_t* __restrict__ cnt) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x)
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
         atomicAdd(&cnt[circle_colour(P, u[e], v[e])], 1);
+        if (v[e] == P) atomicAdd(&cnt[P], 1);
+    }
 }
 
 __global__ void k_colour_keys(int32_t P, const int32_t* __restrict__ ids, int64_t k, const int32_t* __restrict__ u,
@@ -1020,36 +1023,64 @@ __global__ void k_colour_keys(int32_t P, const int32_t* __restrict__ ids, int64_
 
 }  // namespace
 
-// Class sizes of the circle colouring of edges (u, v) into cnt_h [P] (host).
+// Class sizes of the circle colouring of edges (u, v) and, last, the edges at the odd one, into
+// cnt_h [P + 1] (host).
 lowd_status lowd_sys_class_sizes(lowd_ctx* h, const int32_t* u, const int32_t* v, int64_t m, int32_t* cnt_h) {
     const int32_t P = h->n + (h->n & 1) - 1;
     int32_t* cnt = nullptr;
-    LOWD_TRY(dalloc(h, &cnt, P));
-    cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)P, h->st);
+    LOWD_TRY(dalloc(h, &cnt, (size_t)P + 1));
+    cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(int32_t) * ((size_t)P + 1), h->st);
     if (m > 0) LOWD_LAUNCH(k_colour_counts, grid_for(m), kT, 0, h->st, P, u, v, m, cnt);
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(cnt_h, cnt, sizeof(int32_t) * (size_t)P, cudaMemcpyDeviceToHost, h->st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(cnt_h, cnt, sizeof(int32_t) * ((size_t)P + 1), cudaMemcpyDeviceToHost, h->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
     dfree(h, &cnt);
     return e == cudaSuccess ? LOWD_OK : h->fail(e);
 }
 
-// Whether the array serves this graph of C classes.  Its cells grow with n^2, so they are bounded
-// by 2^26 (268 MB: n up to about 11,500 whatever the density) or 16 cells per edge; sparser
-// graphs keep the staged sweep, whose memory grows with the edges.  Measured per class: the array
-// takes 88 (n 129) to 117 ns (n 9,109) for odd n, the one-CTA kernels 148 ns (60 edges a class) to
-// 297 (710) and 933 (2,090), and 310 to 360 below 369 classes, where they keep single FP32 loads.
-// For even n the diagonal is slower (176 to 209 ns; 277 when every row meets the odd one), so from
-// 369 classes on the array takes the graphs whose classes have at least 320 edges: at 232 the
-// staged sweep is still ahead (175 against 203 ns), at 402 it is not (215 against 195; its edges
-// have been read a class early since: 174 -> 159 ns at n 4,048).
-bool lowd_sys_serves(int32_t n, int64_t m, int32_t C, bool pair) {
+// Whether the array serves a graph whose circle colouring has C classes that hold edges, the longest
+// of `longest` edges (padded to 4), `odd_edges` of the edges at the odd one.
+//
+// The array walks all P steps of a pass, the one-CTA kernels the C classes, so what is compared is P
+// times a step with C times a class.  Measured (GB300, random graphs of 71 to 10,002 nodes, ns):
+//  - staged sweep (pair loads), a class: 92 to 105 with up to 128 edges in the longest class, 120 to 136
+//    up to 256, 157 to 170 up to 384, 192 to 201 up to 512 (a warp more per scheduler each time), 222 at
+//    560, 300 to 317 at 770 (weighted 370);
+//  - register ring (single FP32 loads), a class: 290 to 335, above 340 from 64 edges on;
+//  - array, a step, odd n: 110 to 129 with pair loads, 84 to 95 with single ones (165 at 25 nodes, 130
+//    at 33, 110 at 67);
+//  - array, a step, even n, pair loads: 140 with hardly an edge a class, about 180 from 64 edges a class
+//    on (fewer groups without an update), and up to 130 more as more rows meet the odd one (2,048 nodes
+//    of degree 800 203, 770 nodes of degree 640 289); single loads: 430 at 16 nodes, 305 at 32, 205 at 66,
+//    147 at 308, 113 at 2,048 and up to 100 more for the odd one.
+// 10,001 nodes with 300 edges (300 classes): 89 us a pass here against 930 on the array; with 2,500
+// edges 202 against 1,160; 1,030 nodes with 400 edges a class 200 against 289.
+//
+// The cells grow with n^2.  Up to 2^20 of them (4 MB) they may be any number, above it at most 64 per
+// edge, above 2^26 (268 MB, n about 11,500) at most 16: sparser graphs keep the class-major arrays,
+// which grow with the edges.
+bool lowd_sys_serves(int32_t n, int64_t m, int32_t C, int32_t longest, int64_t odd_edges, bool pair) {
+    const Geo g = make_geo(n);
+    const int64_t x = C > 0 ? m / C : 0;   // edges a class
+    int64_t step, cls;
+    if (pair) {
+        cls = 62 + 34 * (((int64_t)longest + 127) / 128);
+        step = (n & 1) ? 120 : 150 + 40 * (x < 64 ? x : 64) / 64 + 130 * odd_edges / n;
+    } else {
+        cls = 300;
+        step = (n & 1) ? 90 + 1500 / n : 120 + 6000 / n + 100 * odd_edges / n;
+    }
+    return lowd_sys_may_serve(n, m) && (int64_t)g.P * step < (int64_t)C * cls;
+}
+
+// What is known before the classes are counted.  (With fewer than P / 3 edges there are fewer classes than
+// that, at 300 ns each at most: a longer class is paid for by the classes its edges do not fill.)
+bool lowd_sys_may_serve(int32_t n, int64_t m) {
     if (n < 9) return false;
     const Geo g = make_geo(n);
-    if (g.KL > lowd_device_sms() * kPairs) return false;
     const int64_t cells = g.steps() << 5;
-    if (cells > ((int64_t)1 << 26) && cells > 16 * m) return false;
-    return (n & 1) != 0 || !pair || m >= 320 * (int64_t)C;
+    if (cells > ((int64_t)1 << 20) && cells > (cells > ((int64_t)1 << 26) ? 16 : 64) * m) return false;
+    return g.KL <= lowd_device_sms() * kPairs && 3 * m >= g.P;
 }
 
 lowd_status lowd_sys_build(lowd_ctx* h, const int32_t* plain_ids, int64_t m_plain, const float* init_splits_canon) {
