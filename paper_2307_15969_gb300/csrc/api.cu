@@ -60,6 +60,18 @@ cudaMemPool_t lowd_pool() {
     return pools[dev];
 }
 
+void lowd_drop_schedule(lowd_ctx* h, lowd_schedule* s) {
+    dfree(h, &s->perm); dfree(h, &s->coff); dfree(h, &s->coff_real); dfree(h, &s->cuv); dfree(h, &s->crk);
+    dfree(h, &s->cw); dfree(h, &s->cs); dfree(h, &s->l); dfree(h, &s->l_lo);
+    dfree(h, &s->s2_ctab); dfree(h, &s->s2_beg); dfree(h, &s->s2_ea); dfree(h, &s->s2_eb);
+    dfree(h, &s->s2_srcA); dfree(h, &s->s2_srcB); dfree(h, &s->s2_lp); dfree(h, &s->s2_blob); dfree(h, &s->s2_blobo);
+    dfree(h, &s->s2_prev); dfree(h, &s->s2_nodes);
+    dfree(h, &s->sys_cs); dfree(h, &s->sys_cw); dfree(h, &s->sys_ids); dfree(h, &s->sys_streams);
+    dfree(h, &s->star_step_seg); dfree(h, &s->star_seg_beg); dfree(h, &s->star_seg_hub); dfree(h, &s->star_bbuf);
+    free(s->coff_h);
+    *s = lowd_schedule();
+}
+
 namespace {
 
 lowd_status check_handle(lowd_handle h) { return h ? LOWD_OK : LOWD_ERR_INVALID_ARG; }
@@ -77,21 +89,13 @@ lowd_status to_caller(lowd_ctx* h, T* dst, const T* src_dev, size_t n) {
 void free_all(lowd_ctx* h) {
     dfree(h, &h->u); dfree(h, &h->v); dfree(h, &h->w); dfree(h, &h->wu); dfree(h, &h->map);
     dfree(h, &h->sort_perm); dfree(h, &h->removal_round);
-    dfree(h, &h->perm); dfree(h, &h->coff); dfree(h, &h->coff_real); dfree(h, &h->cuv); dfree(h, &h->crk);
-    dfree(h, &h->cw); dfree(h, &h->cs); dfree(h, &h->l); dfree(h, &h->l_lo);
-    dfree(h, &h->s2_ctab); dfree(h, &h->s2_beg); dfree(h, &h->s2_ea); dfree(h, &h->s2_eb);
-    dfree(h, &h->s2_srcA); dfree(h, &h->s2_srcB); dfree(h, &h->s2_lp); dfree(h, &h->s2_blob); dfree(h, &h->s2_blobo);
-    dfree(h, &h->s2_prev); dfree(h, &h->s2_nodes);
-    dfree(h, &h->sys_cs); dfree(h, &h->sys_cw); dfree(h, &h->sys_ids); dfree(h, &h->sys_streams);
-    dfree(h, &h->star_step_seg); dfree(h, &h->star_seg_beg); dfree(h, &h->star_seg_hub); dfree(h, &h->star_bbuf);
+    lowd_drop_schedule(h, h);
     if (h->tmp) cudaFree(h->tmp);   // the sort scratch is a plain allocation (need_tmp)
     h->tmp = nullptr;
     h->tmp_cap = 0;
     dfree(h, &h->d_stats); dfree(h, &h->d_i64); dfree(h, &h->d_i32);
     if (h->h_pin) cudaFreeHost(h->h_pin);
     h->h_pin = nullptr;
-    free(h->coff_h);
-    h->coff_h = nullptr;
 }
 
 __global__ void k_init_loads(const int32_t* __restrict__ u, const int32_t* __restrict__ v,

@@ -16,42 +16,10 @@
 // Largest graph (nodes) lowd_extract_noalloc accepts.
 #define LOWD_NOALLOC_MAX_NODES 65536
 
-struct lowd_ctx {
-    cudaStream_t st = nullptr;
-    int mem = LOWD_MEM_HOST;
-    int flags = 0;
-    char err[256] = {0};
-
-    // loaded graph G
-    int32_t n0 = 0;
-    int64_t m0 = 0;
-    int64_t dup = 0;
-    int weighted = 0;
-    int inexact = 0;  // some input weight was off the 2^-20 grid (allowed by flag)
-
-    // current graph (G, or H after pruning): canonical order, lo < hi
-    int32_t n = 0;
-    int64_t m = 0;
-    int32_t* u = nullptr;
-    int32_t* v = nullptr;
-    float* w = nullptr;     // [m] weights, null for unit weights
-    int64_t* wu = nullptr;  // [m] weight units of 2^-20, null for unit weights
-    int32_t* map = nullptr; // [n] current id -> original id; null while current == G
-    int32_t max_deg = -1;      // maximum unweighted degree of the current graph; -1: not computed yet
-
-    // pruning record (original numbering)
-    int pruned = 0;
-    int32_t prune_rounds = 0;
-    int32_t* sort_perm = nullptr;      // [n0]
-    int32_t* removal_round = nullptr;  // [n0]
-
-    // LOWD state, kept in schedule (class-major) order
+// The schedule of a handle's current graph and the LOWD state in its order.
+struct lowd_schedule {
     int inited = 0;
-    int32_t iters = 0;
     int sched = 0;             // 1 one-CTA shared memory, 2 grid matchings
-    int sweep_kernel = 0;      // kernel of the last pass (lowd_info.sweep_kernel)
-    int sweep_E = 0;           // edges per consumer thread of the staged sweep
-    int32_t wave_blocks = 0;   // blocks of the last wavefront pass (0: another kernel ran it)
     int32_t C = 0;             // number of classes
     int64_t m_pad = 0;         // class-major length, each class padded to a multiple of 4
     int32_t* perm = nullptr;   // [m_pad] class-major position -> canonical edge id, -1 = padding
@@ -61,7 +29,6 @@ struct lowd_ctx {
     uint32_t* cuv = nullptr;   // [m_pad] packed ends (lo | hi << 16); padding: (n | n << 16)
     uint32_t* crk = nullptr;   // [m_pad] rank of each end among its node's updates per pass
                                // (16 bits per end, bit 15 = the node's last update)
-    int use_versions = 0;      // 1: the staged sweep uses per-node versions (kernel 5)
     float* cw = nullptr;       // [m_pad] weights (weighted only); padding 0
     float* cs = nullptr;       // [m_pad] splits f_e(lo); padding 0
     float* l = nullptr;        // [n + 1] loads; slot n is the padding sentinel
@@ -96,7 +63,6 @@ struct lowd_ctx {
     int64_t* s2_blobo = nullptr;  // [NC + 1] word offsets of the chunk blobs
     // hub stars (block updates of the edges with exactly one end of degree >= tau), both
     // schedules: the star edges follow the plain ones, at positions [star_p0, star_p0 + star_m)
-    int32_t hub_tau = 0;              // asked for: 0 off, 1 automatic threshold, >= 2 the threshold
     int32_t star_tau = 0;             // threshold in use (0: no star edges)
     int32_t star_S = 0;               // star steps per pass
     int32_t star_nseg = 0;            // stars over all steps
@@ -107,6 +73,44 @@ struct lowd_ctx {
     int32_t* star_seg_beg = nullptr;  // [star_nseg + 1] position of each star's first edge
     int32_t* star_seg_hub = nullptr;  // [star_nseg] hub of each star
     float2* star_bbuf = nullptr;      // [star_m] (a_j, t_j) of stars too large for registers
+};
+
+struct lowd_ctx : lowd_schedule {
+    cudaStream_t st = nullptr;
+    int mem = LOWD_MEM_HOST;
+    int flags = 0;
+    char err[256] = {0};
+
+    // loaded graph G
+    int32_t n0 = 0;
+    int64_t m0 = 0;
+    int64_t dup = 0;
+    int weighted = 0;
+    int inexact = 0;  // some input weight was off the 2^-20 grid (allowed by flag)
+
+    // current graph (G, or H after pruning): canonical order, lo < hi
+    int32_t n = 0;
+    int64_t m = 0;
+    int32_t* u = nullptr;
+    int32_t* v = nullptr;
+    float* w = nullptr;     // [m] weights, null for unit weights
+    int64_t* wu = nullptr;  // [m] weight units of 2^-20, null for unit weights
+    int32_t* map = nullptr; // [n] current id -> original id; null while current == G
+    int32_t max_deg = -1;      // maximum unweighted degree of the current graph; -1: not computed yet
+
+    // pruning record (original numbering)
+    int pruned = 0;
+    int32_t prune_rounds = 0;
+    int32_t* sort_perm = nullptr;      // [n0]
+    int32_t* removal_round = nullptr;  // [n0]
+
+    // what lowd_iterate was asked for, and what it ran
+    int32_t hub_tau = 0;       // hub stars asked for: 0 off, 1 automatic threshold, >= 2 the threshold
+    int use_versions = 0;      // 1: the staged sweep uses per-node versions (kernel 5)
+    int32_t iters = 0;
+    int sweep_kernel = 0;      // kernel of the last pass (lowd_info.sweep_kernel)
+    int sweep_E = 0;           // edges per consumer thread of the staged sweep
+    int32_t wave_blocks = 0;   // blocks of the last wavefront pass (0: another kernel ran it)
 
     // scratch
     void* tmp = nullptr;
@@ -170,6 +174,9 @@ inline void dfree(lowd_ctx* h, T** p) {
     if (*p) cudaFreeAsync(*p, h->st);
     *p = nullptr;
 }
+
+// Frees a schedule's arrays and empties it.
+void lowd_drop_schedule(lowd_ctx* h, lowd_schedule* s);
 
 // bytes to allocate for a radix sort + scans over n elements
 size_t lowd_sort_tmp_bytes(int64_t n);

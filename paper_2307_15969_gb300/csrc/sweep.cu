@@ -1191,31 +1191,33 @@ static lowd_status prepare_schedule(lowd_ctx* h, int schedule_req, const float* 
 
 // Per-node versions (kernel 5) read the class-major arrays: a graph held in the systolic array
 // moves there, once, keeping its splits (its loads are re-derived from them, as after every call).
+// The array is kept until the new schedule stands: without the memory for both the passes go on in it.
 static lowd_status leave_systolic(lowd_ctx* h) {
     float* s = nullptr;
-    LOWD_TRY(dalloc(h, &s, h->m));
-    lowd_status r = lowd_sweep_splits_canonical(h, s);
+    lowd_status r = dalloc(h, &s, h->m);
+    if (r == LOWD_OK) r = lowd_sweep_splits_canonical(h, s);
     if (r == LOWD_OK) {
-        dfree(h, &h->sys_cs); dfree(h, &h->sys_cw); dfree(h, &h->sys_ids); dfree(h, &h->sys_streams);
-        dfree(h, &h->perm); dfree(h, &h->coff); dfree(h, &h->coff_real); dfree(h, &h->cuv);
-        dfree(h, &h->cw); dfree(h, &h->cs); dfree(h, &h->l); dfree(h, &h->l_lo);
-        dfree(h, &h->star_step_seg); dfree(h, &h->star_seg_beg); dfree(h, &h->star_seg_hub); dfree(h, &h->star_bbuf);
-        free(h->coff_h);
-        h->coff_h = nullptr;
-        h->sys = 0;
-        h->sys_m = 0;
-        h->inited = 0;
+        lowd_schedule held = *h;
+        static_cast<lowd_schedule&>(*h) = lowd_schedule();
         r = prepare_schedule(h, 1, s, false);
+        if (r == LOWD_OK) {
+            lowd_drop_schedule(h, &held);
+        } else {
+            lowd_drop_schedule(h, h);
+            static_cast<lowd_schedule&>(*h) = held;
+        }
     }
     cudaStreamSynchronize(h->st);
     dfree(h, &s);
-    return r;
+    return r == LOWD_ERR_OUT_OF_MEMORY ? LOWD_OK : r;
 }
 
 // Build the schedule and its arrays, then initialise the splits (equal split, or the given
-// canonical-order splits) and the loads.
+// canonical-order splits) and the loads.  A preparation that fails leaves nothing behind.
 lowd_status lowd_sweep_prepare(lowd_ctx* h, int schedule_req, const float* init_splits_canon) {
-    return prepare_schedule(h, schedule_req, init_splits_canon, true);
+    const lowd_status r = prepare_schedule(h, schedule_req, init_splits_canon, true);
+    if (r != LOWD_OK) lowd_drop_schedule(h, h);
+    return r;
 }
 
 static lowd_status prepare_schedule(lowd_ctx* h, int schedule_req, const float* init_splits_canon, bool systolic) {
