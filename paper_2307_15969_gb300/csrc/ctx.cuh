@@ -205,7 +205,6 @@ lowd_status lowd_sys_build(lowd_ctx* h, const int32_t* plain_ids, int64_t m_plai
 lowd_status lowd_sys_rederive(lowd_ctx* h, double* L64);
 lowd_status lowd_sys_to_canonical(lowd_ctx* h, float* out);
 lowd_status lowd_sys_from_canonical(lowd_ctx* h, const float* in);
-lowd_status lowd_sys_edge_order(lowd_ctx* h, int32_t* out);
 cudaError_t lowd_sys_passes(lowd_ctx* h, int32_t passes);
 
 // stars.cu

@@ -50,18 +50,20 @@ inline unsigned grid_for(int64_t n) { return lowd_grid_for(n, kT); }
 constexpr int kRankBits = 16;  // rank inside a (class, group, bank) bucket: < 2^16
 constexpr int kBankBits = 4;   // 16 load slots of 8 bytes span the 32 four-byte banks
 
-__global__ void k_circle_colour(const int32_t* __restrict__ u, const int32_t* __restrict__ v, int64_t m,
-                                int32_t n, uint64_t* __restrict__ key, int32_t* __restrict__ val) {
+__global__ void k_circle_colour(const int32_t* __restrict__ ids, int64_t k, const int32_t* __restrict__ u,
+                                const int32_t* __restrict__ v, int32_t n, uint64_t* __restrict__ key,
+                                int32_t* __restrict__ val) {
     const uint32_t Np = (uint32_t)(n + (n & 1));
     const uint32_t P = Np - 1;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
-         e += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t e = ids ? ids[i] : (int32_t)i;
         const uint32_t a = (uint32_t)u[e], b = (uint32_t)v[e];
         const uint32_t c = (b == Np - 1) ? (2u * a) % P : (a + b) % P;
         const uint32_t g = (b != Np - 1 && a + b >= P) ? 1u : 0u;
-        key[e] = ((uint64_t)c << (kBankBits + 1)) | ((uint64_t)g << kBankBits) |
+        key[i] = ((uint64_t)c << (kBankBits + 1)) | ((uint64_t)g << kBankBits) |
                  (uint64_t)(a & ((1u << kBankBits) - 1u));
-        val[e] = (int32_t)e;
+        val[i] = e;
     }
 }
 
@@ -100,12 +102,6 @@ __global__ void k_pad_sizes(const int32_t* __restrict__ coff_real, int32_t C, in
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < C;
          c += (int64_t)gridDim.x * blockDim.x)
         pcnt[c] = (coff_real[c + 1] - coff_real[c] + 3) & ~3;
-}
-
-// x[i] = ids[x[i]]: indices into a subset of the edges -> edge ids
-__global__ void k_subset_to_ids(const int32_t* __restrict__ ids, int64_t k, int32_t* __restrict__ x) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k; i += (int64_t)gridDim.x * blockDim.x)
-        x[i] = ids[x[i]];
 }
 
 __global__ void k_fill_perm(int32_t* __restrict__ perm_pad, int64_t m_pad) {
@@ -1134,6 +1130,25 @@ cudaError_t run_passes(lowd_ctx* h, int32_t passes) {
 
 }  // namespace
 
+// The edges (ids null: all k, else the k listed) in class-major order: keys, the class above the lowest
+// kRankBits + kBankBits + 1 bits, and edge ids.  key, val: two buffers of k entries each.
+static void class_major(lowd_ctx* h, const int32_t* ids, int64_t k, uint64_t* const key[2], int32_t* const val[2],
+                        uint64_t** kout, int32_t** vout) {
+    cudaStream_t st = h->st;
+    LOWD_LAUNCH(k_circle_colour, grid_for(k), kT, 0, st, ids, k, h->u, h->v, h->n, key[0], val[0]);
+    const uint32_t P = (uint32_t)(h->n + (h->n & 1)) - 1u;
+    const int cbits = bit_length_u64(P > 0 ? P - 1 : 0);
+    const int cur = radix_sort_pairs<uint64_t, int32_t>(key[0], val[0], key[1], val[1], k, cbits + kBankBits + 1, h->tmp, st);
+    uint64_t* kA = key[cur];
+    int32_t* vA = val[cur];
+    uint64_t* kB = key[1 - cur];
+    int32_t* vB = val[1 - cur];
+    LOWD_LAUNCH(k_bank_rounds, grid_for(k), kT, 0, st, kA, k, kB);
+    const int r2 = radix_sort_pairs<uint64_t, int32_t>(kB, vA, kA, vB, k, cbits + kBankBits + 1 + kRankBits, h->tmp, st);
+    *kout = r2 ? kA : kB;
+    *vout = r2 ? vB : vA;
+}
+
 // The schedule as the systolic array holds it, if it serves these edges (*built): class sizes
 // and offsets, the cells, and the class-major arrays for the star edges alone.  The loads are
 // pairs exactly where the staged sweep would run (single FP32 loads otherwise, as in the
@@ -1259,8 +1274,6 @@ static lowd_status prepare_schedule(lowd_ctx* h, int schedule_req, const float* 
             }
         }
         const int64_t mc = sp.pid ? sp.m_plain : m;   // edges the colouring covers
-        const int32_t* cu = sp.pid ? sp.gu : h->u;
-        const int32_t* cv = sp.pid ? sp.gv : h->v;
         if ((s = h->need_tmp(lowd_sort_tmp_bytes(m > n ? m : n)))) break;
         if ((s = dalloc(h, &key[0], m))) break;
         if ((s = dalloc(h, &key[1], m))) break;
@@ -1269,23 +1282,10 @@ static lowd_status prepare_schedule(lowd_ctx* h, int schedule_req, const float* 
         if ((s = dalloc(h, &head, m))) break;
         if ((s = dalloc(h, &hpos, m))) break;
         int32_t C = 0;
-        int cur = 0;
         uint64_t* kfin = key[0];
         int32_t* vfin = val[0];
         if (mc > 0) {
-            LOWD_LAUNCH(k_circle_colour, grid_for(mc), kT, 0, st, cu, cv, mc, n, key[0], val[0]);
-            const uint32_t P = (uint32_t)(n + (n & 1)) - 1u;
-            const int cbits = bit_length_u64(P > 0 ? P - 1 : 0);
-            cur = radix_sort_pairs<uint64_t, int32_t>(key[0], val[0], key[1], val[1], mc, cbits + kBankBits + 1, h->tmp, st);
-            uint64_t* kA = key[cur];
-            int32_t* vA = val[cur];
-            uint64_t* kB = key[1 - cur];
-            int32_t* vB = val[1 - cur];
-            LOWD_LAUNCH(k_bank_rounds, grid_for(mc), kT, 0, st, kA, mc, kB);
-            const int r2 = radix_sort_pairs<uint64_t, int32_t>(kB, vA, kA, vB, mc, cbits + kBankBits + 1 + kRankBits, h->tmp, st);
-            kfin = r2 ? kA : kB;
-            vfin = r2 ? vB : vA;
-            if (sp.pid) LOWD_LAUNCH(k_subset_to_ids, grid_for(mc), kT, 0, st, sp.pid, mc, vfin);
+            class_major(h, sp.pid, mc, key, val, &kfin, &vfin);
             LOWD_LAUNCH(k_class_heads, grid_for(mc), kT, 0, st, kfin, mc, kRankBits + kBankBits + 1, head);
             scan_exclusive<int32_t>(head, hpos, mc, h->d_i32 + 5, h->tmp, st);
             if (cudaMemcpyAsync(h->h_pin, h->d_i32 + 5, sizeof(int32_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -1382,13 +1382,28 @@ lowd_status lowd_sweep_load_canonical(lowd_ctx* h, const float* splits_dev) {
 
 // The update order as canonical edge ids (padding removed) into out_dev [m].
 lowd_status lowd_sweep_edge_order(lowd_ctx* h, int32_t* out_dev) {
-    if (h->sys) {   // the plain classes, then the star edges (no padding)
-        LOWD_TRY(lowd_sys_edge_order(h, out_dev));
-        if (h->m_pad > 0)
-            LOWD_CK(cudaMemcpyAsync(out_dev + h->sys_m, h->perm, sizeof(int32_t) * (size_t)h->m_pad,
-                                    cudaMemcpyDeviceToDevice, h->st));
-        LOWD_CK(cudaStreamSynchronize(h->st));
-        return LOWD_OK;
+    if (h->sys) {   // the plain classes, in the order of the class-major arrays, then the star edges (no padding)
+        uint64_t* key[2] = {nullptr, nullptr};
+        int32_t* val[2] = {nullptr, nullptr};
+        const int64_t k = h->sys_m;
+        lowd_status r = h->need_tmp(lowd_sort_tmp_bytes(k));
+        for (int i = 0; i < 2 && r == LOWD_OK; ++i)
+            if ((r = dalloc(h, &key[i], k)) == LOWD_OK) r = dalloc(h, &val[i], k);
+        cudaError_t e = cudaSuccess;
+        if (r == LOWD_OK && k > 0) {
+            uint64_t* kfin;
+            int32_t* vfin;
+            class_major(h, h->sys_ids, k, key, val, &kfin, &vfin);
+            e = cudaGetLastError();
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(out_dev, vfin, sizeof(int32_t) * (size_t)k, cudaMemcpyDeviceToDevice, h->st);
+        }
+        if (r == LOWD_OK && e == cudaSuccess && h->m_pad > 0)
+            e = cudaMemcpyAsync(out_dev + k, h->perm, sizeof(int32_t) * (size_t)h->m_pad, cudaMemcpyDeviceToDevice, h->st);
+        const cudaError_t es = cudaStreamSynchronize(h->st);
+        if (e == cudaSuccess) e = es;
+        for (int i = 0; i < 2; ++i) { dfree(h, &key[i]); dfree(h, &val[i]); }
+        return r != LOWD_OK ? r : (e != cudaSuccess ? h->fail(e) : LOWD_OK);
     }
     int32_t *f = nullptr, *pos = nullptr;
     LOWD_TRY(h->need_tmp(lowd_sort_tmp_bytes(h->m_pad)));

@@ -1012,15 +1012,6 @@ __global__ void k_colour_counts(int32_t P, const int32_t* __restrict__ u, const 
     }
 }
 
-__global__ void k_colour_keys(int32_t P, const int32_t* __restrict__ ids, int64_t k, const int32_t* __restrict__ u,
-                              const int32_t* __restrict__ v, uint32_t* __restrict__ key, int32_t* __restrict__ val) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t e = ids ? ids[i] : (int32_t)i;
-        key[i] = (uint32_t)circle_colour(P, u[e], v[e]);
-        val[i] = e;
-    }
-}
-
 }  // namespace
 
 // Class sizes of the circle colouring of edges (u, v) and, last, the edges at the odd one, into
@@ -1129,30 +1120,6 @@ lowd_status lowd_sys_from_canonical(lowd_ctx* h, const float* in) {
                     h->v, h->w, in, false, h->sys_cs, h->sys_cw);
     LOWD_CK_LAUNCH();
     return LOWD_OK;
-}
-
-// The plain edges in the order a pass updates them: by class, then by edge id.
-lowd_status lowd_sys_edge_order(lowd_ctx* h, int32_t* out) {
-    const int64_t m = h->sys_m;
-    if (m == 0) return LOWD_OK;
-    const int32_t P = h->n + (h->n & 1) - 1;
-    uint32_t* key[2] = {nullptr, nullptr};
-    int32_t* val[2] = {nullptr, nullptr};
-    lowd_status s = h->need_tmp(lowd_sort_tmp_bytes(m));
-    for (int i = 0; i < 2 && s == LOWD_OK; ++i) {
-        s = dalloc(h, &key[i], m);
-        if (s == LOWD_OK) s = dalloc(h, &val[i], m);
-    }
-    if (s == LOWD_OK) {
-        LOWD_LAUNCH(k_colour_keys, grid_for(m), kT, 0, h->st, P, h->sys_ids, m, h->u, h->v, key[0], val[0]);
-        const int cur = radix_sort_pairs<uint32_t, int32_t>(key[0], val[0], key[1], val[1], m,
-                                                            bit_length_u64((uint64_t)P), h->tmp, h->st);
-        cudaError_t e = cudaMemcpyAsync(out, val[cur], sizeof(int32_t) * (size_t)m, cudaMemcpyDeviceToDevice, h->st);
-        if (e == cudaSuccess) e = cudaGetLastError();
-        if (e != cudaSuccess) s = h->fail(e);
-    }
-    for (int i = 0; i < 2; ++i) { dfree(h, &key[i]); dfree(h, &val[i]); }
-    return s;
 }
 
 // T passes over the plain edges.
