@@ -471,6 +471,14 @@ uint64_t lowd_launch_count(void);
  * LOWD_ERR_CUDA if it could not run.  Uses the default stream.  No counterpart in the paper. */
 lowd_status lowd_selftest_barrier_timeout(int32_t* err_bits);
 
+/* The same for the bounded waits of the pass kernels whose blocks wait for one another's values:
+ * which = 0, the wavefronts (two blocks of the nine a graph takes: the rest never hand on their
+ * columns); which = 1, the leading classes of the level order (an edge waits for an update that
+ * never comes).  With short limits the waits must expire, set their bit of the error word (0: value 8,
+ * 1: value 2) and end the kernel.  text (may be NULL) receives what lowd_last_error would say of it,
+ * at most capacity bytes with the terminating zero.  Status codes as above. */
+lowd_status lowd_selftest_pass_timeout(int32_t which, int32_t* err_bits, char* text, int32_t capacity);
+
 #ifdef __cplusplus
 }
 #endif

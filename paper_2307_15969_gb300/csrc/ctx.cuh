@@ -16,6 +16,12 @@
 // Largest graph (nodes) lowd_extract_noalloc accepts.
 #define LOWD_NOALLOC_MAX_NODES 65536
 
+// Error word of a pass (bits).
+constexpr int32_t kStagedExpired = 1;    // a bounded wait on a staged copy or a node version expired
+constexpr int32_t kGridExpired = 2;      // a grid barrier or a wait on another block's node entry did
+constexpr int32_t kBadDescriptor = 4;    // a read descriptor pointed outside the stages
+constexpr int32_t kWaveExpired = 8;      // a wait of the wavefronts expired
+
 // The schedule of a handle's current graph and the LOWD state in its order.
 struct lowd_schedule {
     int inited = 0;
@@ -206,6 +212,7 @@ lowd_status lowd_sys_rederive(lowd_ctx* h, double* L64);
 lowd_status lowd_sys_to_canonical(lowd_ctx* h, float* out);
 lowd_status lowd_sys_from_canonical(lowd_ctx* h, const float* in);
 cudaError_t lowd_sys_passes(lowd_ctx* h, int32_t passes);
+cudaError_t lowd_sys_selftest(int32_t* err_bits);
 
 // stars.cu
 struct StarSplit {
@@ -226,6 +233,7 @@ cudaError_t lowd_star_pass(lowd_ctx* h);
 lowd_status lowd_stream_prepare(lowd_ctx* h, const float* init_splits_canon);
 lowd_status lowd_stream_rederive(lowd_ctx* h, double* L64);
 cudaError_t lowd_stream_passes(lowd_ctx* h, int32_t passes);
+cudaError_t lowd_nodes_selftest(int32_t* err_bits);
 
 // api.cu
 lowd_status lowd_apply_splits_dev(lowd_ctx* h, const float* splits_canon_dev);

@@ -857,7 +857,7 @@ template <bool WEIGHTED>
 __global__ void __launch_bounds__(512)
 k_sweep_nodes(int32_t beg, int32_t end, const int32_t* __restrict__ ea, const int32_t* __restrict__ eb,
               const uint2* __restrict__ prev, const float* __restrict__ cw, float* __restrict__ cs,
-              ulonglong2* __restrict__ nodes, int32_t* __restrict__ err) {
+              ulonglong2* __restrict__ nodes, uint32_t most_polls, int32_t* __restrict__ err) {
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     // consecutive warps of the order lie on different SMs
@@ -898,9 +898,9 @@ k_sweep_nodes(int32_t beg, int32_t end, const int32_t* __restrict__ ea, const in
             ++polls;
             if ((polls & 1023u) == 0u) {
                 bool stop = *(volatile int32_t*)err != 0;
-                if (polls >= kFlowPolls) {
+                if (polls >= most_polls) {
                     stop = true;
-                    if (lane == 0) atomicOr(err, 2);
+                    if (lane == 0) atomicOr(err, kGridExpired);
                 }
                 if (__any_sync(0xffffffffu, stop)) return;
             }
@@ -1244,7 +1244,8 @@ cudaError_t lowd_stream_passes(lowd_ctx* h, int32_t passes) {
             const float* pcw = h->cw;
             float* pcs = h->cs;
             ulonglong2* pn = h->s2_nodes;
-            void* args[] = {&beg, &end, &pea, &peb, &pp, &pcw, &pcs, &pn, &errp};
+            uint32_t polls = kFlowPolls;
+            void* args[] = {&beg, &end, &pea, &peb, &pp, &pcw, &pcs, &pn, &polls, &errp};
             const cudaError_t r = cudaLaunchCooperativeKernel((const void*)gk, dim3(lowd_device_sms()),
                                                               dim3(kFlowThreads[g]), args, 0, h->st);
             lowd_note_launch();
@@ -1272,4 +1273,37 @@ cudaError_t lowd_stream_passes(lowd_ctx* h, int32_t passes) {
     if (e != cudaSuccess) return e;
     LOWD_LAUNCH(k_unpack_loads, grid_for(h->n), kT, 0, h->st, h->s2_lp, h->n, h->l, h->l_lo);
     return cudaGetLastError();
+}
+
+// One edge whose update before it, by its record, never comes.
+cudaError_t lowd_nodes_selftest(int32_t* err_bits) {
+    struct Host {
+        ulonglong2 nodes[2];
+        uint2 prev;
+        int32_t ea, eb;
+        float cs;
+        int32_t err;
+    } x = {};
+    x.prev = make_uint2(7u, 7u);
+    x.eb = 1;
+    x.cs = 0.5f;
+    Host* d = nullptr;
+    cudaError_t e = cudaMalloc((void**)&d, sizeof(Host));
+    if (e != cudaSuccess) return e;
+    e = cudaMemcpy(d, &x, sizeof(x), cudaMemcpyHostToDevice);
+    int32_t beg = 0, end = 1;
+    const int32_t *ea = &d->ea, *eb = &d->eb;
+    const uint2* prev = &d->prev;
+    const float* cw = nullptr;
+    float* cs = &d->cs;
+    ulonglong2* nodes = d->nodes;
+    uint32_t polls = 1u << 12;
+    int32_t* err = &d->err;
+    void* args[] = {&beg, &end, &ea, &eb, &prev, &cw, &cs, &nodes, &polls, &err};
+    if (e == cudaSuccess)
+        e = cudaLaunchCooperativeKernel((const void*)k_sweep_nodes<false>, dim3(1), dim3(32), args, 0, nullptr);
+    lowd_note_launch();
+    if (e == cudaSuccess) e = cudaMemcpy(err_bits, &d->err, sizeof(int32_t), cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    return e;
 }

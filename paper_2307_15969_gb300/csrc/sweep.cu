@@ -1421,6 +1421,25 @@ lowd_status lowd_sweep_edge_order(lowd_ctx* h, int32_t* out_dev) {
     return s;
 }
 
+static const char* pass_error(int32_t bits) {
+    if (bits & kBadDescriptor) return "sweep: a read descriptor pointed outside the stages";
+    if (bits & kWaveExpired) return "sweep: a bounded wait of the wavefronts expired";
+    if (bits & kGridExpired) return "sweep: a bounded wait across the grid expired";
+    return "sweep: a bounded wait on a staged copy expired";
+}
+
+extern "C" lowd_status lowd_selftest_pass_timeout(int32_t which, int32_t* err_bits, char* text, int32_t capacity) {
+    if (which < 0 || which > 1 || !err_bits || (text && capacity < 1)) return LOWD_ERR_INVALID_ARG;
+    *err_bits = 0;
+    const cudaError_t e = which == 0 ? lowd_sys_selftest(err_bits) : lowd_nodes_selftest(err_bits);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? LOWD_ERR_OUT_OF_MEMORY : LOWD_ERR_CUDA;
+    }
+    if (text) snprintf(text, (size_t)capacity, "%s", *err_bits ? pass_error(*err_bits) : "");
+    return LOWD_OK;
+}
+
 lowd_status lowd_sweep_run(lowd_ctx* h, int32_t k, const lowd_options* opt, lowd_stats* out) {
     lowd_options o;
     memset(&o, 0, sizeof(o));
@@ -1447,10 +1466,7 @@ lowd_status lowd_sweep_run(lowd_ctx* h, int32_t k, const lowd_options* opt, lowd
         LOWD_CK(cudaStreamSynchronize(h->st));
         const int32_t kerr = *(int32_t*)(h->h_pin + 8);
         if (kerr != 0) {
-            snprintf(h->err, sizeof(h->err), "%s",
-                     (kerr & 4) ? "sweep: a read descriptor pointed outside the stages"
-                                : ((kerr & 2) ? "sweep: a bounded wait across the grid expired"
-                                              : "sweep: a bounded wait on a staged copy expired"));
+            snprintf(h->err, sizeof(h->err), "%s", pass_error(kerr));
             return LOWD_ERR_CUDA;
         }
         done += step;

@@ -122,7 +122,8 @@ struct SysArgs {
     ulonglong2* in_low;       // [grid][P + kPad] streams into each block's first low tile (block 0: the wrap)
     ulonglong2* in_high;      // [grid][P + kPad]
     ulonglong2* in_odd;       // [grid] the odd one's load
-    int32_t* err;        // bit 0: a wait expired (every warp then leaves)
+    int32_t* err;        // kWaveExpired: a wait expired (every warp then leaves)
+    uint32_t spin_shift; // the waits' limits are divided by 2 to this power
 };
 
 // A stream entry: (hi, tag), (lo, tag).  Each 8-byte half is written and read as one access and
@@ -310,9 +311,9 @@ struct Bad {
     __device__ __forceinline__ bool expired(uint32_t spins, uint32_t limit) const {
         if ((spins & 255u) != 255u) return false;
         if (*flag) return true;
-        if (spins >= limit || *(volatile int32_t*)a->err != 0) {
+        if (spins >= (limit >> a->spin_shift) || *(volatile int32_t*)a->err != 0) {
             *flag = 1;
-            atomicOr(a->err, 1);
+            atomicOr(a->err, kWaveExpired);
             return true;
         }
         return false;
@@ -1180,6 +1181,7 @@ cudaError_t lowd_sys_passes(lowd_ctx* h, int32_t passes) {
         a.in_high = h->sys_streams + (size_t)grid * pitch;
         a.in_odd = h->sys_streams + 2 * (size_t)grid * pitch;
         a.err = h->d_i32 + 8;
+        a.spin_shift = 0;
         void* args[] = {&a};
         e = cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(32 * (2 * W + (grid > 1 ? 2 : 0))), args, smem,
                                         h->st);
@@ -1187,5 +1189,44 @@ cudaError_t lowd_sys_passes(lowd_ctx* h, int32_t passes) {
         h->sys_tag += (uint32_t)(k + 2) * lapt;
         done += k;
     }
+    return e;
+}
+
+// Two blocks of the nine that 1,031 nodes take, with short limits: the columns that the others would
+// hand on never come, so the waits expire (the streams are as long as for all nine).
+cudaError_t lowd_sys_selftest(int32_t* err_bits) {
+    const Geo g = make_geo(1031);
+    const size_t pitch = (size_t)g.P + kPad, cells = (size_t)g.steps() << 5;
+    const size_t blocks = (size_t)(g.KL + kPairsOdd - 1) / kPairsOdd;
+    const size_t streams = 2 * blocks * pitch + blocks;
+    const size_t smem = (size_t)(2 * kPairsOdd + 1) * kRing * 16u + (size_t)kPairsOdd * (kOddBytes + 16u) +
+                        (size_t)kPairsOdd * 2u * kCellBytes;
+    unsigned char* d = nullptr;
+    cudaError_t e = cudaMalloc((void**)&d, 16 * streams + 4 * (cells + 2 * (size_t)g.n + 1));
+    if (e != cudaSuccess) return e;
+    SysArgs a;
+    a.g = g;
+    a.W = kPairsOdd;
+    a.T = 2;
+    a.odd = 0;
+    a.tag0 = (uint32_t)pitch;
+    a.in_low = reinterpret_cast<ulonglong2*>(d);
+    a.in_high = a.in_low + blocks * pitch;
+    a.in_odd = a.in_low + 2 * blocks * pitch;
+    a.cs = reinterpret_cast<float*>(d + 16 * streams);
+    a.cw = nullptr;
+    a.l = a.cs + cells;
+    a.l_lo = a.l + g.n;
+    a.err = reinterpret_cast<int32_t*>(a.l_lo + g.n);
+    a.spin_shift = 7;
+    void* args[] = {&a};
+    auto kern = k_sweep_systolic<true, false, false>;
+    e = cudaMemset(d, 0, 16 * streams + 4 * (cells + 2 * (size_t)g.n + 1));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)
+        e = cudaLaunchCooperativeKernel((const void*)kern, dim3(2), dim3(32 * (2 * kPairsOdd + 2)), args, smem, nullptr);
+    lowd_note_launch();
+    if (e == cudaSuccess) e = cudaMemcpy(err_bits, a.err, sizeof(int32_t), cudaMemcpyDeviceToHost);
+    cudaFree(d);
     return e;
 }

@@ -39,7 +39,7 @@ EXPORTED = (
     "lowd_ldd_dks_bound", "lowd_mpnn_param_count", "lowd_mpnn_create", "lowd_mpnn_set_params",
     "lowd_mpnn_get_params", "lowd_mpnn_bind", "lowd_mpnn_set_features", "lowd_mpnn_forward", "lowd_mpnn_backward", "lowd_mpnn_adam",
     "lowd_mpnn_read", "lowd_warm_start", "lowd_mpnn_last_error", "lowd_mpnn_free",
-    "lowd_selftest_barrier_timeout",
+    "lowd_selftest_barrier_timeout", "lowd_selftest_pass_timeout",
 )
 LOWD_MPNN_SIGMA = 1
 LOWD_MPNN_LOADS = 2
@@ -160,6 +160,8 @@ def load_library(path: str = LIB_PATH):
     lib.lowd_launch_count.argtypes = []
     lib.lowd_selftest_barrier_timeout.restype = i32
     lib.lowd_selftest_barrier_timeout.argtypes = [C.POINTER(i32)]
+    lib.lowd_selftest_pass_timeout.restype = i32
+    lib.lowd_selftest_pass_timeout.argtypes = [i32, C.POINTER(i32), C.c_char_p, i32]
     lib.lowd_batch_create.restype = i32
     lib.lowd_batch_create.argtypes = [i32, P, P, P, P, i32, P, C.POINTER(P)]
     lib.lowd_batch_run.restype = i32
@@ -196,6 +198,15 @@ def lowd_selftest_barrier_timeout():
     bits = C.c_int32()
     s = load_library().lowd_selftest_barrier_timeout(C.byref(bits))
     return s, bits.value
+
+
+def lowd_selftest_pass_timeout(which: int):
+    """The expiry path of the pass kernels' waits between blocks (see include/lowd.h); returns
+    (status, error word, message)."""
+    bits = C.c_int32()
+    text = C.create_string_buffer(256)
+    s = load_library().lowd_selftest_pass_timeout(int(which), C.byref(bits), text, 256)
+    return s, bits.value, text.value.decode()
 
 
 def _is_torch(x) -> bool:
