@@ -449,20 +449,31 @@ __device__ __forceinline__ void poll_entry(const Tile& t, int32_t s, const Bad& 
     }
 }
 
-// until the entries j0 .. j1 - 1 of the group at step s0 (EDGE: those that exist) are in t.e.  The tag
-// of every one of them is looked at: they mostly come in order, so it is the last one that is
-// polled, but the wrap's come from the warps of different tiles, and nothing orders those.
+// until the entries j0 .. j1 - 1 of the group at step s0 are in t.e.  They mostly come in order, so the last
+// one is polled; but the wrap's come from the warps of different tiles, and nothing orders those: where the
+// group is not whole then, its entries are polled one after the other.  (An entry that every lane has seen
+// stays until this tile has told that it read it.)  Without a loop around the polls, each of which is
+// bounded, a group costs least: n 9,109 at density 0.156 1,014 us a pass (a counted loop 1,061, or 1,090 where
+// the clipping below was part of it), 6,193 weighted 714 (746, 775).
+template <bool PAIR>
+__device__ __forceinline__ void await_group(Tile& t, int32_t s0, int j0, int j1, const Bad& w, bool& bad) {
+    if (__all_sync(0xffffffffu, missing<PAIR>(t, s0, j0, j1) == 0u)) return;
+    poll_entry<PAIR>(t, s0 + j1 - 1, w, bad);
+    read_ahead<PAIR>(t, s0);
+    if (__all_sync(0xffffffffu, missing<PAIR>(t, s0, j0, j1) == 0u)) return;
+#pragma unroll 1
+    for (int j = j0; j < j1 - 1; ++j) poll_entry<PAIR>(t, s0 + j, w, bad);
+    read_ahead<PAIR>(t, s0);
+}
+
+// the same, for those of the entries that exist (EDGE: the inputs may run out inside the group)
 template <bool PAIR, bool EDGE>
 __device__ __forceinline__ void await_entries(Tile& t, int32_t s0, int j0, int j1, const Bad& w, bool& bad) {
-    if (EDGE) {                            // the inputs may run out inside the group
-        j1 = min(j1, t.in_end - s0);
-        if (j1 <= j0) return;
+    if (EDGE && s0 + j1 > t.in_end) {
+        if (s0 + j0 < t.in_end) await_group<PAIR>(t, s0, j0, t.in_end - s0, w, bad);
+        return;
     }
-    for (uint32_t spins = 1; __any_sync(0xffffffffu, missing<PAIR>(t, s0, j0, j1) != 0u) && !bad; ++spins) {
-        poll_entry<PAIR>(t, s0 + j1 - 1, w, bad);
-        read_ahead<PAIR>(t, s0);
-        if ((spins & 255u) == 255u) bad = __any_sync(0xffffffffu, bad || w.expired(spins, kSpinSmem));
-    }
+    await_group<PAIR>(t, s0, j0, j1, w, bad);
 }
 
 // an entry in a slot of the odd exchange
