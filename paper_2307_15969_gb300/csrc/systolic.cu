@@ -1050,14 +1050,14 @@ lowd_status lowd_sys_class_sizes(lowd_ctx* h, const int32_t* u, const int32_t* v
 //    up to 256, 157 to 170 up to 384, 192 to 201 up to 512 (a warp more per scheduler each time), 222 at
 //    560, 300 to 317 at 770 (weighted 370);
 //  - register ring (single FP32 loads), a class: 290 to 335, above 340 from 64 edges on;
-//  - array, a step, odd n: 110 to 129 with pair loads, 84 to 95 with single ones (165 at 25 nodes, 130
+//  - array, a step, odd n: 107 to 116 with pair loads, 84 to 95 with single ones (168 at 25 nodes, 124
 //    at 33, 110 at 67);
-//  - array, a step, even n, pair loads: 140 with hardly an edge a class, about 180 from 64 edges a class
-//    on (fewer groups without an update), and up to 130 more as more rows meet the odd one (2,048 nodes
-//    of degree 800 203, 770 nodes of degree 640 289); single loads: 430 at 16 nodes, 305 at 32, 205 at 66,
-//    147 at 308, 113 at 2,048 and up to 100 more for the odd one.
-// 10,001 nodes with 300 edges (300 classes): 89 us a pass here against 930 on the array; with 2,500
-// edges 202 against 1,160; 1,030 nodes with 400 edges a class 200 against 289.
+//  - array, a step, even n, pair loads: 140 with hardly an edge a class, about 175 from 64 edges a class
+//    on (more rows with an update in a group), and up to 130 more as more rows meet the odd one (2,048
+//    nodes of degree 800 198, 770 nodes of degree 640 284); single loads: 430 at 16 nodes, 310 at 32, 203
+//    at 66, 140 at 308, 113 at 2,048 and up to 100 more for the odd one.
+// 10,001 nodes with 300 edges (300 classes): 89 us a pass on the register ring, 930 on the array; with
+// 2,500 edges 202 on the staged sweep, 1,100 on the array; 1,030 nodes with 400 edges a class 200 and 292.
 //
 // The cells grow with n^2.  Up to 2^20 of them (4 MB) they may be any number, above it at most 64 per
 // edge, above 2^26 (268 MB, n about 11,500) at most 16: sparser graphs keep the class-major arrays,
@@ -1068,7 +1068,7 @@ bool lowd_sys_serves(int32_t n, int64_t m, int32_t C, int32_t longest, int64_t o
     int64_t step, cls;
     if (pair) {
         cls = 62 + 34 * (((int64_t)longest + 127) / 128);
-        step = (n & 1) ? 120 : 150 + 40 * (x < 64 ? x : 64) / 64 + 130 * odd_edges / n;
+        step = (n & 1) ? 112 : 140 + 40 * (x < 64 ? x : 64) / 64 + 130 * odd_edges / n;
     } else {
         cls = 300;
         step = (n & 1) ? 90 + 1500 / n : 120 + 6000 / n + 100 * odd_edges / n;
@@ -1141,9 +1141,9 @@ cudaError_t lowd_sys_passes(lowd_ctx* h, int32_t passes) {
     const bool pair = h->sys_pair != 0;
     // One block when the pairs fit it (every stream then stays in shared memory).  Of several, two
     // pairs each for odd n while every SM holds one: fewer warps per SM are faster steps, more
-    // blocks are more slow hops.  Two against four pairs: n 513 59 against 64 us, 1,031 114 (124),
-    // 4,047 457 (489), weighted 460 (498), 9,109 1,066 (1,136); one pair 6 to 10 % slower than two.
-    // Even n gains nothing (770: 238 against 232 us, 9,110: 1,828 against 1,829) and keeps four.
+    // blocks are more slow hops.  Two against four pairs: n 513 57 against 60 us, 1,031 111 (121),
+    // 4,047 437 (469), 6,193 weighted 718 (756), 9,109 1,015 (1,074); one pair 6 to 10 % slower than
+    // two.  Even n gains nothing (770: 238 against 232 us, 9,110: 1,828 against 1,829) and keeps four.
     const int several = (g.P == h->n && g.KL <= lowd_device_sms() * kPairsOdd) ? kPairsOdd : kPairs;
     const int W = g.KL <= (weighted ? kPairs : kMaxW) ? g.KL : several;
     const int grid = (g.KL + W - 1) / W;
