@@ -53,12 +53,13 @@ def _peaks():
     return 6800.0, "fallback"
 
 
-# per pass kernel of schedule 1: its source file, the spans hashed (kernel and launcher, to its
-# closing brace) and its committed ncu record
+# per pass kernel of schedule 1: its source file, the spans hashed (layout, kernel with all that it
+# calls, and launcher to its closing brace) and its committed ncu record
 RECORDS = {
     "k_sweep_tma": ("sweep.cu", (("struct TmaLayout {", "// The same staging as k_sweep_tma"),
                                  ("cudaError_t launch_sweep_tma(", "\n}\n")), "k_sweep_tma_rmat22_dram.json"),
-    "k_sweep_systolic": ("systolic.cu", (("k_sweep_systolic(const SysArgs a) {", "\n}\n"),
+    "k_sweep_systolic": ("systolic.cu", (("constexpr int kPairs = ", "// ---------------------------------"
+                                          "--------------------------------- building and reading the cells"),
                                          ("cudaError_t lowd_sys_passes(", "\n}\n")),
                          "k_sweep_systolic_rmat22_dram.json"),
 }
