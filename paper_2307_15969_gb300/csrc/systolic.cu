@@ -40,14 +40,12 @@
 // shared memory keeps them there for the launch.
 //
 // What bounds it: a chain of P steps per pass, not bandwidth (DRAM 0.3 TB/s on the scale-22 R-MAT
-// core).  A step's own chain is a shuffle and a transfer (81 cycles for pair loads, alone on an
-// SM; 130 with the cells, streams and stores around it, 160 with eight warps on the SM); on the
-// critical path lie the steps at the diagonal and the right edge (150 to 190), a lag of about
-// three steps per tile, since inputs are checked four at a time, and the way between blocks.
-// Measured (GB300, per pass, against the one-CTA sweep of one barrier per class): n 9,109,
-// 6.25 M edges 1,066 us (was 2,705); n 9,110 1,807 us (2,705); n 4,047 457 us (701); n 6,193
-// weighted 736 us (1,189); n 307 29 us (111); n 71 7.9 us (22);
-// G(4400, 0.95) 1,218 us (4,106).
+// core).  A step's own chain is a shuffle and a transfer; on the critical path, about 230 cycles a
+// step, lie the steps at the diagonal and the right edge, a lag of about three steps per tile, since
+// inputs are checked four at a time, and the way between blocks.
+// Measured (GB300, per pass, against the one-CTA sweep of one barrier per class): scale-22 R-MAT core, n
+// 9,109, 6.49 M edges 1,027 us (2,705); n 9,110 at density 0.156 1,898 (2,890); n 4,047 at 0.126 437
+// (701); n 6,193 weighted at 0.08 718 (1,189); n 307 27 (111); n 71 7.4 (22).
 #include "ctx.cuh"
 #include "prims.cuh"
 #include "async.cuh"
