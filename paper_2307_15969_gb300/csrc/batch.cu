@@ -668,7 +668,7 @@ cudaError_t prepare(const lowd_batch_options& o, int32_t count, LaunchCfg* cfg) 
     const int per = o.ctas_per_sm;
     int smem = (optin - 2048) / per - 1024;
     smem &= ~1023;
-    e = cudaFuncSetAttribute(k_batch_lowd, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e = lowd_allow_smem(k_batch_lowd, (size_t)((optin - 2048 - 1024) & ~1023));   // that of one CTA per SM
     if (e != cudaSuccess) return e;
     cfg->smem = smem;
     cfg->threads = o.threads;

@@ -25,7 +25,7 @@ constexpr int32_t kWaveExpired = 8;      // a wait of the wavefronts expired
 // The schedule of a handle's current graph and the LOWD state in its order.
 struct lowd_schedule {
     int inited = 0;
-    int sched = 0;             // 1 one-CTA shared memory, 2 grid matchings
+    int sched = 0;             // 1 circle colouring, 2 level order
     int32_t C = 0;             // number of classes
     int64_t m_pad = 0;         // class-major length, each class padded to a multiple of 4
     int32_t* perm = nullptr;   // [m_pad] class-major position -> canonical edge id, -1 = padding
@@ -179,6 +179,14 @@ template <class T>
 inline void dfree(lowd_ctx* h, T** p) {
     if (*p) cudaFreeAsync(*p, h->st);
     *p = nullptr;
+}
+
+// Lets `kern` be launched with up to `most` bytes of dynamic shared memory.  Every call for a kernel gives
+// the same limit, not the size of the launch to come: another thread that needs less could lower that
+// between this call and the launch.
+template <class K>
+inline cudaError_t lowd_allow_smem(K kern, size_t most) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
 // Frees a schedule's arrays and empties it.

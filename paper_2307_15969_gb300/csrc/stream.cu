@@ -287,6 +287,7 @@ constexpr int kWbShift = 21;
 enum { WB_ALWAYS = 0, WB_NEVER = 1, WB_LAST_PASS = 2 };
 constexpr uint32_t kZeroSlot = 0;   // ring offset of an always-zero load (padding ends)
 constexpr uint32_t kRingHead = 128; // stages start here
+constexpr size_t kStreamSmemMost = 226 * 1024;   // dynamic shared memory at most: 227 KB less the static barriers
 
 constexpr int kSegs = 64;           // classes (or class pieces) per chunk
 constexpr int kHdrInts = 68;        // chunk header: begin, padded size, segment count, 64 ends, pad
@@ -1022,7 +1023,7 @@ lowd_status lowd_stream_prepare(lowd_ctx* h, const float* init_splits_canon) {
             int32_t* errp = h->d_i32 + 10;
             cudaMemsetAsync(errp, 0, sizeof(int32_t), st);
             void* args[] = {&pend, &succ, &level, &fr[0], &fr[1], &ctl, &errp};
-            cudaError_t e = cudaFuncSetAttribute(k_levels, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLevelSmem);
+            cudaError_t e = lowd_allow_smem(k_levels, kLevelSmem);
             if (e == cudaSuccess)
                 e = cudaLaunchCooperativeKernel((const void*)k_levels, dim3(lowd_device_sms()), dim3(kLevelT), args,
                                                 kLevelSmem, st);
@@ -1063,7 +1064,7 @@ lowd_status lowd_stream_prepare(lowd_ctx* h, const float* init_splits_canon) {
         if (cudaMemcpyAsync(coff.data(), h->coff_real, sizeof(int32_t) * ((size_t)C + 1), cudaMemcpyDeviceToHost, st) !=
                 cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) { s = h->fail(cudaGetLastError()); break; }
         const int32_t D = kLead, S = 2 * kLead;
-        const size_t budget = 227 * 1024 - kRingHead - 1024;
+        const size_t budget = kStreamSmemMost - kRingHead;
         const uint32_t E = stream_edges_per_stage(S, weighted, budget);
         // header rows: [0] padded begin, [1] padded size, [2] segments, [3 + g] end of segment
         // g relative to the begin; real_beg: the chunk's first real (unpadded) position
@@ -1217,7 +1218,7 @@ cudaError_t lowd_stream_passes(lowd_ctx* h, int32_t passes) {
     const StreamLayout L = stream_layout((uint32_t)h->s2_E, weighted);
     const size_t smem = kRingHead + (size_t)L.bytes * (size_t)h->s2_S;
     auto kern = weighted ? k_sweep_stream<true> : k_sweep_stream<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = lowd_allow_smem(kern, kStreamSmemMost);
     if (e != cudaSuccess) return e;
     h->sweep_kernel = 4;
     h->sweep_E = 0;

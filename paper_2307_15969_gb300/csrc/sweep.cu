@@ -954,7 +954,7 @@ cudaError_t launch_sweep_tma(lowd_ctx* h, int32_t passes, int32_t maxlen, bool* 
     auto kern = E == 4 ? k_sweep_tma<WEIGHTED, 4> : (E == 2 ? k_sweep_tma<WEIGHTED, 2> : k_sweep_tma<WEIGHTED, 1>);
     h->sweep_kernel = 1;
     h->sweep_E = E;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.total);
+    cudaError_t e = lowd_allow_smem(kern, kStagedSmemMost);
     if (e != cudaSuccess) return e;
     const int32_t per = (int32_t)(0x7fffffff / NC);
     for (int32_t done = 0; done < passes && e == cudaSuccess;) {
@@ -1038,7 +1038,7 @@ cudaError_t launch_sweep_flow(lowd_ctx* h, int32_t passes, int32_t maxlen, bool*
     int threads = ((maxlen + 31) / 32) * 32;
     if (threads < 64) threads = 64;
     auto kern = k_sweep_flow<WEIGHTED>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.total);
+    cudaError_t e = lowd_allow_smem(kern, kStagedSmemMost);
     if (e != cudaSuccess) return e;
     h->sweep_kernel = 5;
     h->sweep_E = 1;
@@ -1087,14 +1087,14 @@ cudaError_t launch_sweep(lowd_ctx* h, int32_t passes) {
         auto kern = co_smem ? k_sweep_vec<WEIGHTED, kRing, true> : k_sweep_vec<WEIGHTED, kRing, false>;
         h->sweep_kernel = 2;
         h->sweep_E = 0;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = lowd_allow_smem(kern, budget);
         if (e != cudaSuccess) return e;
         LOWD_LAUNCH(kern, 1, threads, smem, h->st, h->n, h->C, h->coff, cuv, cw, cs, h->l, h->l_lo, passes);
     } else {
         auto kern = k_sweep_simple<WEIGHTED>;
         h->sweep_kernel = 3;
         h->sweep_E = 0;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lbytes);
+        cudaError_t e = lowd_allow_smem(kern, budget);
         if (e != cudaSuccess) return e;
         LOWD_LAUNCH(kern, 1, threads, lbytes, h->st, h->n, h->C, h->coff, cuv, cw, cs, h->l, h->l_lo, passes);
     }

@@ -1158,7 +1158,7 @@ cudaError_t lowd_sys_passes(lowd_ctx* h, int32_t passes) {
                             : (weighted ? k_sweep_systolic<false, true, true> : k_sweep_systolic<false, false, true>))
                     : (pair ? (weighted ? k_sweep_systolic<true, true, false> : k_sweep_systolic<true, false, false>)
                             : (weighted ? k_sweep_systolic<false, true, false> : k_sweep_systolic<false, false, false>));
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = lowd_allow_smem(kern, kSmemMost);
     if (e != cudaSuccess) return e;
     const size_t pitch = (size_t)g.P + kPad;
     const size_t words = (size_t)grid * (2 * pitch + 1);
@@ -1231,7 +1231,7 @@ cudaError_t lowd_sys_selftest(int32_t* err_bits) {
     void* args[] = {&a};
     auto kern = k_sweep_systolic<true, false, false>;
     e = cudaMemset(d, 0, 16 * streams + 4 * (cells + 2 * (size_t)g.n + 1));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = lowd_allow_smem(kern, kSmemMost);
     if (e == cudaSuccess)
         e = cudaLaunchCooperativeKernel((const void*)kern, dim3(2), dim3(32 * (2 * kPairsOdd + 2)), args, smem, nullptr);
     lowd_note_launch();
