@@ -1054,6 +1054,10 @@ lowd_status lowd_stream_prepare(lowd_ctx* h, const float* init_splits_canon) {
             if ((s = dalloc(h, &h->coff_real, (size_t)C + 1))) break;
             LOWD_LAUNCH(k_level_heads, grid_for(m), kT, 0, st, c4 ? k32[1] : k32[0], m, h->coff_real);
             LOWD_LAUNCH(k_fill_i32s, 1, 32, 0, st, h->coff_real + C, (int64_t)1, (int32_t)m);
+            // what the order was made from: the streams below need the most memory
+            ord = nullptr;
+            dfree(h, &deg); dfree(h, &val[0]); dfree(h, &k32[0]); dfree(h, &k32[1]); dfree(h, &k64[0]); dfree(h, &k64[1]);
+            dfree(h, &succ); dfree(h, &pend); dfree(h, &level);
         } else {
             if ((s = dalloc(h, &h->coff_real, 1))) break;
             cudaMemsetAsync(h->coff_real, 0, sizeof(int32_t), st);
@@ -1079,6 +1083,7 @@ lowd_status lowd_stream_prepare(lowd_ctx* h, const float* init_splits_canon) {
             LOWD_LAUNCH(k_previous, grid_for(m_grid), kT, 0, st, ranks, m_grid, pred, pos,
                         reinterpret_cast<uint32_t*>(h->s2_prev));
         }
+        dfree(h, &pred); dfree(h, &pos);
         flow_segments(h, coff, K);
         const int64_t grid_pad = (m_grid + 3) & ~(int64_t)3;
         std::vector<int32_t> ctab, real_beg;
@@ -1154,6 +1159,7 @@ lowd_status lowd_stream_prepare(lowd_ctx* h, const float* init_splits_canon) {
         if (m_pad > 0) {
             if (m_pad_plain > 0) LOWD_LAUNCH(k_fill_i32s, grid_for(m_pad_plain), kT, 0, st, h->perm, m_pad_plain, -1);
             if (m > 0) LOWD_LAUNCH(k_pad_scatter, grid_for(m), kT, 0, st, order, m, m_grid, rb, h->s2_beg, NCp, h->perm);
+            dfree(h, &fr[0]); dfree(h, &fr[1]);   // order and ranks
             LOWD_LAUNCH(k_stream_gather, grid_for(m_pad), kT, 0, st, h->perm, m_pad, n, h->u, h->v, h->w,
                         init_splits_canon, h->s2_ea, h->s2_eb, h->cw, h->cs);
             // ---- 7. descriptors from each node's occurrences (sorted by node, stable in position)
